@@ -230,12 +230,16 @@ lnv_status lnv_plan_destroy(lnv_plan *plan);
  * matrix multiplication of Sec. 3): C = alpha mask_C(op(A) op(B)) + beta C.
  * A_dev, B_dev, C_dev are value arrays in `prec` (double or float) with
  * NSF x NSF blocks, NSF in {1, 2, 4, 9}.  beta = 0: C is overwritten (its
- * old values are not read, NaN included) and nothing is allocated.  beta !=
+ * old values are not read, NaN included) and, kernel 11 on FP64 values aside
+ * (below), nothing is allocated.  beta !=
  * 0: the product is formed in a scratch buffer the context keeps (allocated
  * or grown on the first such call, which then synchronises; later calls of
  * the same size allocate nothing) and combined with C elementwise in FP64
- * arithmetic, rounded to the value precision.  Kernel 11 on FP64 values keeps the
- * digits of A and B in a second such buffer of the context. */
+ * arithmetic, rounded to the value precision.  Kernel 11 on FP64 values takes
+ * memory for the digits of A and B from a stream-ordered pool of the context and
+ * gives it back within the call (in a stream capture both are nodes of the graph,
+ * which then owns the memory); with no room for them it runs kernel 0.  The pool
+ * keeps what was in use at one time until the context goes. */
 lnv_status lnv_bsr_multiply(lnv_ctx *ctx, const lnv_plan *plan, int nsf, lnv_prec prec,
                             const void *A_dev, const void *B_dev, void *C_dev, double alpha,
                             double beta);

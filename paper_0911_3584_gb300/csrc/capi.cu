@@ -133,12 +133,13 @@ WsLayout ws_layout(const lnv_system *s, int with_grad)
     // FP64 products on the tensor cores: digits of the smaller operand (S, H, L; X
     // too with 9 x 9 blocks, whose digits are longer than they are), the rows'
     // magnitudes, and with 9 x 9 blocks digits of the larger operand (with 4 x 4 they
-    // go where an intermediate is not alive; see lnv_energy_grad)
+    // go where an intermediate is not alive, see lnv_energy_grad; S's and H's where T is
+    // to come, if they fit there: with T truncated below r_sh they do not)
     const bool dig = (s->nsf == 4 || s->nsf == 9) && s->prec == LNV_FP64, dig9 = dig && s->nsf == 9;
     const size_t d_sh = dig_bytes(s->P_sh, s->nsf), d_l = dig_bytes(s->P_l, s->nsf), d_x = dig_bytes(s->P_x, s->nsf),
                  d_t = dig_bytes(s->P_t, s->nsf);
     L.D = dig ? take(std::max({d_sh, d_l, dig9 ? d_x : (size_t)0})) : 0;
-    L.E = dig9 ? take(std::max({d_sh, d_x, d_t})) : 0;
+    L.E = dig9 ? take(std::max({d_sh, d_x, d_t})) : dig && s->P_sh->nnzb > s->P_t->nnzb ? take(d_sh) : 0;
     L.head = dig ? take(dig_head_bytes(s->n, s->nsf)) : 0;
     L.total = off;
     return L;
@@ -204,6 +205,17 @@ lnv_status lnv_ctx_create(int device, void *cuda_stream, lnv_ctx **out)
         set_error("context status word: %s", cudaGetErrorString(e));
         return e == cudaErrorMemoryAllocation ? LNV_ERR_OOM : LNV_ERR_CUDA;
     }
+    int pools = 0;
+    if (cudaDeviceGetAttribute(&pools, cudaDevAttrMemoryPoolsSupported, device) == cudaSuccess && pools) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        uint64_t keep = UINT64_MAX;  // until the context goes: as much as was in use at one time
+        if (cudaMemPoolCreate(&c->dig_pool, &props) != cudaSuccess) c->dig_pool = nullptr;
+        else cudaMemPoolSetAttribute(c->dig_pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    }
+    cudaGetLastError();  // a device without pools is no error
     *out = c;
     return LNV_OK;
 }
@@ -240,7 +252,7 @@ lnv_status lnv_ctx_destroy(lnv_ctx *ctx)
     if (ctx) {
         cudaFree(ctx->scratch);
         cudaFree(ctx->prod_scratch);
-        cudaFree(ctx->dig_scratch);
+        if (ctx->dig_pool) cudaMemPoolDestroy(ctx->dig_pool);
         cudaFree(ctx->dev_status);
     }
     delete ctx;
@@ -573,7 +585,8 @@ lnv_status lnv_system_autotune(lnv_ctx *ctx, lnv_system *sys, const void *S_dev,
     LNV_ARG(sys && S_dev && H_dev && L_dev, "null pointer");
     LNV_ARG(aligned16(S_dev) && aligned16(H_dev) && aligned16(L_dev), "value arrays must be 16-byte aligned");
     if (reps < 1) reps = 1;
-    const size_t dig_held = ctx->dig_scratch_bytes;
+    uint64_t dig_held = 0;
+    if (ctx->dig_pool) LNV_CUDA(cudaMemPoolGetAttribute(ctx->dig_pool, cudaMemPoolAttrReservedMemCurrent, &dig_held));
     // one evaluation fills the intermediates the products read
     const WsLayout wl = ws_layout(sys, 1);
     void *G = nullptr;
@@ -665,8 +678,8 @@ lnv_status lnv_system_autotune(lnv_ctx *ctx, lnv_system *sys, const void *S_dev,
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     cudaStreamSynchronize(ctx->stream);
-    // the candidates' digit buffers: evaluations use the workspace instead
-    if (ctx->dig_scratch_bytes > dig_held) dig_scratch_free(ctx);
+    // the memory of the candidates' digits is given back: evaluations use the workspace
+    if (ctx->dig_pool) cudaMemPoolTrimTo(ctx->dig_pool, (size_t)dig_held);
     cudaFree(G);
     cudaFree(out);
     return st;
@@ -791,9 +804,9 @@ lnv_status lnv_energy_grad(lnv_ctx *ctx, lnv_system *sys, const void *S_dev, con
     sys->profiled_grad = grad;
     // FP64 products on the tensor cores: the digits of S, H or L in D, those of
     // the larger operand in the buffer of an intermediate that is not alive.
-    auto digits = [&](const lnv_plan *pl, void *a, void *b, bool fits) {
+    auto digits = [&](const lnv_plan *pl, void *a, void *b) {
         DigScratch d;
-        if (plan_digits(pl, nsf, pr) && (fits || nsf == 9)) {
+        if (plan_digits(pl, nsf, pr)) {
             d.a = nsf == 9 ? ws + wl.D : a;
             d.b = nsf == 9 ? ws + wl.E : b;
             d.head = (int *)(ws + wl.head);
@@ -808,10 +821,10 @@ lnv_status lnv_energy_grad(lnv_ctx *ctx, lnv_system *sys, const void *S_dev, con
         LNV_CUDA(cudaMemsetAsync(ws + wl.head, 0, dig_zero_bytes(), ctx->stream));
     LNV_TRY(mark(0));
     // a1: X = L S, Y = L H (S's, then H's digits where T comes later)
-    LNV_TRY(product(sys->pl_xy, digits(sys->pl_xy, D, T, sys->P_sh->nnzb <= sys->P_t->nnzb), L_dev, S_dev, H_dev, X, Y));
+    LNV_TRY(product(sys->pl_xy, digits(sys->pl_xy, D, sys->P_sh->nnzb <= sys->P_t->nnzb ? T : ws + wl.E), L_dev, S_dev, H_dev, X, Y));
     LNV_TRY(mark(1));
     // a2: T = S X (= SLS), U = S Y (= SLH) (X's, then Y's digits where Z comes later)
-    const DigScratch d_tu = digits(sys->pl_tu, D, Z, true);
+    const DigScratch d_tu = digits(sys->pl_tu, D, Z);
     if (grad) LNV_TRY(product(sys->pl_tu, d_tu, S_dev, X, Y, T, U));
     else LNV_TRY(product(sys->pl_tu, d_tu, S_dev, X, nullptr, T, nullptr));
     // Z and W on digits overwrite T, which dN_e/dL reads on L's pattern: its
@@ -820,7 +833,7 @@ lnv_status lnv_energy_grad(lnv_ctx *ctx, lnv_system *sys, const void *S_dev, con
     if (t_early) LNV_TRY(sub_blocks(ctx, sys->P_l, sys->sub_lt, nsf, pr, T, GN_dev));
     LNV_TRY(mark(2));
     // a3: Z = L T (= LSLS) on R_X (T's digits replace T)
-    DigScratch d_z = digits(sys->pl_z, D, T, true);
+    DigScratch d_z = digits(sys->pl_z, D, T);
     d_z.b_finite = plan_digits(sys->pl_tu, nsf, pr);
     LNV_TRY(product(sys->pl_z, d_z, L_dev, T, nullptr, Z, nullptr));
     LNV_TRY(mark(3));
@@ -833,12 +846,12 @@ lnv_status lnv_energy_grad(lnv_ctx *ctx, lnv_system *sys, const void *S_dev, con
     if (grad) {
         // a6: Q = H Z (= HLSLS) on R_L;  a5: W = X^T U^T (= SLHLS) on R_L
         // (Z's and X's digits where Y was, U's where T was)
-        const DigScratch d_q = digits(sys->pl_q, D, Y, true);
+        const DigScratch d_q = digits(sys->pl_q, D, Y);
         LNV_TRY(product(sys->pl_q, d_q, H_dev, Z, nullptr, Q, nullptr));
         // V = S Z (= SLSLS) on R_L has the patterns of Q = H Z
         if (GN_dev) LNV_TRY(product(sys->pl_q, d_q, S_dev, Z, nullptr, V, nullptr));
         LNV_TRY(mark(5));
-        LNV_TRY(product(sys->pl_w, digits(sys->pl_w, Y, T, true), X, U, nullptr, W, nullptr));
+        LNV_TRY(product(sys->pl_w, digits(sys->pl_w, Y, T), X, U, nullptr, W, nullptr));
         LNV_TRY(mark(6));
         // a7: G = 6(U + U^T) - 4(Q^T + W + Q) on L's pattern
         LNV_TRY(grad_assemble(ctx, sys->P_l, sys->sub_lt, sys->w_map, nsf, pr, U, W, Q, G_dev));
@@ -848,7 +861,7 @@ lnv_status lnv_energy_grad(lnv_ctx *ctx, lnv_system *sys, const void *S_dev, con
         LNV_TRY(mark(7));
     } else if (GN_dev) {
         // a7 (electron count): dN_e/dL = 12 (SLS - SLSLS) on L's pattern
-        LNV_TRY(product(sys->pl_q, digits(sys->pl_q, D, Y, true), S_dev, Z, nullptr, V, nullptr));
+        LNV_TRY(product(sys->pl_q, digits(sys->pl_q, D, Y), S_dev, Z, nullptr, V, nullptr));
         LNV_TRY(grad_ne_assemble(ctx, sys->P_l, t_early ? nullptr : sys->sub_lt, nsf, pr, t_early ? GN_dev : T, V,
                                  GN_dev));
     }

@@ -71,8 +71,9 @@ struct lnv_ctx {
     size_t scratch_n = 0;
     void *prod_scratch = nullptr;  // product of lnv_bsr_multiply with beta != 0 (grown on demand)
     size_t prod_scratch_bytes = 0;
-    void *dig_scratch = nullptr;  // operand digits of FP64 products on the tensor cores (grown on demand)
-    size_t dig_scratch_bytes = 0;
+    // stream-ordered pool of the operand digits of FP64 products outside an evaluation
+    // (null: the device has none, such products are formed term by term)
+    cudaMemPool_t dig_pool = nullptr;
 };
 
 struct lnv_pattern {
@@ -315,7 +316,6 @@ inline bool plan_digits(const lnv_plan *pl, int nsf, lnv_prec prec)
 // reuse_a: a and head hold A's digits and magnitudes of the call before.
 lnv_status launch_umma64(lnv_ctx *ctx, const lnv_plan *pl, int nsf, bool upper, const void *A, const void *B, void *C,
                          const DigScratch &s, bool reuse_a);
-void dig_scratch_free(lnv_ctx *ctx);
 void tile_plan_free(TilePlan *tt);
 lnv_status scan_exclusive(cudaStream_t st, const int64_t *in, int64_t n, int64_t *out);
 void group_plan_free(GroupPlan *gp);
@@ -326,7 +326,8 @@ lnv_status pattern_host_cols(lnv_ctx *ctx, const lnv_pattern *p);
 lnv_status multiply(lnv_ctx *ctx, const lnv_plan *plan, int nsf, lnv_prec prec, const void *A,
                     const void *B, void *C);
 // Two products sharing A and the patterns of B and C: C1 = A B1, C2 = A B2.
-// dig: the digit buffers of a plan with plan_digits (null: the context's own).
+// dig: the digit buffers of a plan with plan_digits (null: taken from the context's pool
+// for the call).
 lnv_status multiply2(lnv_ctx *ctx, const lnv_plan *plan, int nsf, lnv_prec prec, const void *A,
                      const void *B1, const void *B2, void *C1, void *C2, const DigScratch *dig = nullptr);
 

@@ -1,13 +1,15 @@
 """FP64 digit products (kernel 11 on FP64 values, kernel 10 on those of 9 x 9 systems) at the limits of their
-operands: NaN and infinities met while the operands are split, results at the ends of the exponent range."""
+operands: NaN and infinities met while the operands are split, results at the ends of the exponent range, buffers of
+the digits that outlive a call."""
 from fractions import Fraction
 
 import numpy as np
 import pytest
 import torch
 
-from paper_0911_3584_gb300 import Context, Pattern, Plan
-from tests.gpu_util import to_dev
+import oracle
+from paper_0911_3584_gb300 import Context, Pattern, Plan, System
+from tests.gpu_util import rel_fro, to_dev, workload
 
 pytestmark = pytest.mark.gpu
 
@@ -85,3 +87,90 @@ def test_subnormal_results_are_rounded_once(ctx, k):
     want = float(Fraction(a) * Fraction(b))
     assert want == (p >> k) * 2.0 ** -1074
     assert np.array_equal(C, np.full((1, 4, 4), want)), (C / 2.0 ** -1074, p >> k)
+
+
+def _product(ctx, seed, n, cutoff):
+    rng = np.random.default_rng(seed)
+    P = Pattern.build(ctx, rng.uniform(0, 24.0, size=(n, 3)), np.array([24.0, 24.0, 24.0]), cutoff)
+    plan = Plan(ctx, P, P, P, trans_b=True)
+    plan.set_kernel("tensor-tile")
+    return plan, [to_dev(rng.standard_normal((P.nnzb, 4, 4)), torch.float64, ctx.device) for _ in "ab"]
+
+
+def _tuned_system(ctx):
+    w, S, H, L = workload(2, 4, 6.6, 8.0, 7)
+    sysm = System(ctx, 4, "fp64", w["pos"], w["cell"], 6.6, 8.0)
+    sysm.autotune(*(to_dev(M["val"], torch.float64, ctx.device) for M in (S, H, L)), reps=1)
+
+
+def test_captured_product_outlives_larger_ones(cuda_device):
+    """A product captured in a graph replays with its bits after a larger product and an autotune on the same
+    context, with other arrays allocated and filled in between; it needs no call before the capture."""
+    ctx = Context(cuda_device)
+    plan, (a, b) = _product(ctx, 1, 300, 5.0)
+    C = torch.zeros((plan.C.nnzb, 4, 4), dtype=torch.float64, device=cuda_device)
+    graph, side, old = torch.cuda.CUDAGraph(), torch.cuda.Stream(cuda_device), ctx.stream
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=side):
+        ctx.set_stream(side)
+        try:
+            plan.multiply(a, b, C)
+        finally:
+            ctx.set_stream(old)
+    want = plan.multiply(a, b)
+    big, vals = _product(ctx, 2, 1200, 8.0)
+    big.multiply(*vals)
+    _tuned_system(ctx)
+    torch.cuda.synchronize()
+    junk = [torch.full((1 << 26,), float("nan"), dtype=torch.float64, device=cuda_device) for _ in range(4)]
+    for _ in range(3):
+        C.zero_()
+        graph.replay()
+        big.multiply(*vals)
+        assert torch.equal(C, want)
+    assert all(torch.isnan(j).all() for j in junk)
+    assert ctx.device_status() == 0
+
+
+def test_products_on_two_streams_of_one_context(cuda_device):
+    """Products that take turns on two streams share no buffer."""
+    ctx = Context(cuda_device)
+    cases = [_product(ctx, k, n, 8.0) for k, n in enumerate((900, 700))]
+    want = [plan.multiply(*v) for plan, v in cases]
+    streams, old = [torch.cuda.Stream(cuda_device) for _ in cases], ctx.stream
+    got = [[torch.empty_like(w) for _ in range(6)] for w in want]
+    torch.cuda.synchronize()
+    for i in range(6):
+        for s, (plan, v), g in zip(streams, cases, got):
+            ctx.set_stream(s)
+            plan.multiply(*v, C_vals=g[i])
+    ctx.set_stream(old)
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, w) for g, w in zip(got, want) for x in g)
+    assert ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("nsf", [4, 9])
+def test_truncation_below_the_range_of_s(cuda_device, nsf):
+    """r_t < r_sh: S has more blocks than T, whose place its digits do not fit; equal to the oracle, captured too, with
+    an autotune of another system in between."""
+    ctx = Context(cuda_device)
+    from synth import si_diamond_positions, sym_block_values
+    rng = np.random.default_rng(8)
+    pos, cell = si_diamond_positions(2, rng)
+    r_sh, r_l, r_x, r_t = 6.0, 3.0, 4.0, 4.0
+    pat = {k: oracle.pattern(pos, cell, r) for k, r in (("S", r_sh), ("H", r_sh), ("L", r_l))}
+    M = {k: oracle.csr(*pat[k], sym_block_values(*pat[k], pos, cell, nsf, k, rng)) for k in "SHL"}
+    ref = oracle.lnv_energy_grad_truncated(pos, cell, r_sh, r_l, r_x, r_t, M["S"], M["H"], M["L"])
+    sysm = System(ctx, nsf, "fp64", pos, cell, r_sh, r_l, r_x=r_x, r_t=r_t)
+    vals = [to_dev(M[k]["val"], torch.float64, ctx.device) for k in "SHL"]
+    graph, out, G = sysm.capture(*vals)
+    _tuned_system(ctx)
+    for _ in range(2):
+        out.zero_()
+        G.zero_()
+        graph.replay()
+        assert abs(out[0, 0].item() - ref["E"]) <= 1e-12 * abs(ref["E"])
+        assert abs(out[0, 1].item() - ref["Ne"]) <= 1e-12 * abs(ref["Ne"])
+        assert rel_fro(G.cpu().numpy(), ref["G"]) <= 1e-13
+    assert ctx.device_status() == 0
