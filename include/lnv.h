@@ -55,7 +55,17 @@ typedef int lnv_status;
 #define LNV_ERR_TIMEOUT (-6)     /* a bounded device-side wait ran out (see
                                     lnv_ctx_device_status)                  */
 
-/* Arithmetic of a call.  LNV_FP64: values, products and sums in FP64.
+/* Arithmetic of a call.  LNV_FP64: values and sums in FP64; products in FP64, or in
+ * exact digits of operands scaled to 55 bits per row of op(A) and column of op(B)
+ * (kernels 10 and 11 of lnv_plan_info, with which a system's 4 x 4 and 9 x 9 products
+ * begin).  Plain FP64 products are within K 2^-53 sum_k |a_ik b_kj| of the exact ones (K
+ * terms), digit products within K 2^-53 max|row i of op(A)| max|column j of op(B)|.  A row
+ * or a column that is not finite, or whose largest element meets no element of the
+ * other operand within 2^-4 of the largest of its own column or row (as when the
+ * inner index is badly scaled), is formed term by term in FP64 all the same: so in the
+ * largest element of every row and column both bounds are of one size, and E, N_e and G do not
+ * depend on the scale of the basis functions.  Single elements far below those of their
+ * row and column hold fewer bits; lnv_system_set_stage_kernel selects plain products.
  * LNV_FP32: values stored and multiplied in FP32 with FP32 accumulation of
  * the block products; traces, energies and the gradient combination are
  * accumulated in FP64 from the FP32 operands. */
@@ -200,10 +210,9 @@ lnv_status lnv_plan_product(lnv_ctx *ctx, const lnv_pattern *A, const lnv_patter
  * that are sparse as a whole but dense per tile (T = SX, U = SY); either
  * op(B); a symmetric first output is formed on the tiles of its upper part
  * and mirrored; FP32 values with NSF = 4, and FP64 values with NSF = 4 through
- * exact 8-bit digits of operands scaled per row and column (the error is
- * relative to the largest elements of op(A)'s row and op(B)'s column and below
- * that of a plain FP64 sum of terms of that size; operands with NaN or infinity
- * are multiplied term by term; other cases run kernel 0), 12
+ * exact 8-bit digits of operands scaled per row and column (its bound and
+ * the rows and columns that are formed term by term: see LNV_FP64; other cases
+ * run kernel 0), 12
  * and 13 the single-pass forms of 9 and 11: operands rounded to TF32 (round
  * to nearest), one MMA per K step, FP32 accumulation, no low parts; their
  * error (about 1e-4 relative) misses the FP32-level bound, so the

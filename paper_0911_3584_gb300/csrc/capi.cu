@@ -96,6 +96,8 @@ struct lnv_system {
     int profile = 0;
     int profiled_grad = 0;
     cudaEvent_t ev[kStages + 1] = {};
+    cudaEvent_t ev_u = nullptr;  // after U, where it is formed after Z (profiled_u)
+    bool profiled_u = false;
 };
 
 namespace {
@@ -124,22 +126,25 @@ WsLayout ws_layout(const lnv_system *s, int with_grad)
     L.X = take(s->P_x->nnzb * bs);
     L.Y = take(s->P_x->nnzb * bs);
     L.Z = take(s->P_x->nnzb * bs);
-    L.T = take(s->P_t->nnzb * bs);
-    L.U = with_grad ? take(s->P_t->nnzb * bs) : 0;
+    // FP64 products on the tensor cores: digits of the smaller operand (S, H, L; X
+    // too with 9 x 9 blocks, whose digits are longer than they are) and the rows'
+    // magnitudes; with 9 x 9 blocks digits of the larger operand too.  With 4 x 4 blocks,
+    // whose digits are as long as they are, these go where an intermediate is not alive
+    // (see lnv_energy_grad): those of S, H, Y and U to T, which they may not fit if T is
+    // truncated, those of T to U, which is needed for this without the gradient too, and
+    // those of L to V, which comes last.
+    const bool dig = (s->nsf == 4 || s->nsf == 9) && s->prec == LNV_FP64, dig9 = dig && s->nsf == 9, dig4 = dig && !dig9;
+    const int64_t n_t = dig4 ? std::max({s->P_t->nnzb, s->P_x->nnzb, s->P_sh->nnzb}) : s->P_t->nnzb;
+    L.T = take(n_t * bs);
+    L.U = with_grad || dig4 ? take(s->P_t->nnzb * bs) : 0;
     L.W = with_grad ? take(s->P_lu->nnzb * bs) : 0;
     L.Q = with_grad ? take(s->P_l->nnzb * bs) : 0;
     L.V = take(s->P_l->nnzb * bs);  // S Z for dN_e/dL
     L.rows = take(sizeof(double) * 4 * (size_t)std::max<int64_t>(s->n, 1));
-    // FP64 products on the tensor cores: digits of the smaller operand (S, H, L; X
-    // too with 9 x 9 blocks, whose digits are longer than they are), the rows'
-    // magnitudes, and with 9 x 9 blocks digits of the larger operand (with 4 x 4 they
-    // go where an intermediate is not alive, see lnv_energy_grad; S's and H's where T is
-    // to come, if they fit there: with T truncated below r_sh they do not)
-    const bool dig = (s->nsf == 4 || s->nsf == 9) && s->prec == LNV_FP64, dig9 = dig && s->nsf == 9;
     const size_t d_sh = dig_bytes(s->P_sh, s->nsf), d_l = dig_bytes(s->P_l, s->nsf), d_x = dig_bytes(s->P_x, s->nsf),
                  d_t = dig_bytes(s->P_t, s->nsf);
-    L.D = dig ? take(std::max({d_sh, d_l, dig9 ? d_x : (size_t)0})) : 0;
-    L.E = dig9 ? take(std::max({d_sh, d_x, d_t})) : dig && s->P_sh->nnzb > s->P_t->nnzb ? take(d_sh) : 0;
+    L.D = dig9 ? take(std::max({d_sh, d_l, d_x})) : dig ? take(d_sh) : 0;
+    L.E = dig9 ? take(std::max({d_sh, d_x, d_t})) : 0;
     L.head = dig ? take(dig_head_bytes(s->n, s->nsf)) : 0;
     L.total = off;
     return L;
@@ -158,6 +163,7 @@ void system_free(lnv_system *s)
     cudaFree(s->io_dev);
     for (auto &e : s->ev)
         if (e) cudaEventDestroy(e);
+    if (s->ev_u) cudaEventDestroy(s->ev_u);
     delete s;
 }
 
@@ -712,6 +718,7 @@ lnv_status lnv_system_profile(lnv_system *sys, int enable)
     if (enable)
         for (auto &e : sys->ev)
             if (!e) LNV_CUDA(cudaEventCreate(&e));
+    if (enable && !sys->ev_u) LNV_CUDA(cudaEventCreate(&sys->ev_u));
     sys->profile = enable ? 1 : 0;
     return LNV_OK;
 }
@@ -729,6 +736,13 @@ lnv_status lnv_system_stage_ms(lnv_system *sys, double *ms)
             LNV_CUDA(cudaEventElapsedTime(&f, sys->ev[k], sys->ev[k + 1]));
             ms[k] = f;
         }
+    }
+    if (sys->profiled_u) {
+        // between the traces and Q: U's time belongs to T and U
+        float f = 0.f;
+        LNV_CUDA(cudaEventElapsedTime(&f, sys->ev[4], sys->ev_u));
+        ms[1] += f;
+        ms[4] -= f;
     }
     return LNV_OK;
 }
@@ -803,39 +817,49 @@ lnv_status lnv_energy_grad(lnv_ctx *ctx, lnv_system *sys, const void *S_dev, con
     };
     sys->profiled_grad = grad;
     // FP64 products on the tensor cores: the digits of S, H or L in D, those of
-    // the larger operand in the buffer of an intermediate that is not alive.
-    auto digits = [&](const lnv_plan *pl, void *a, void *b) {
+    // the larger operand in the buffer of an intermediate that is not alive (the
+    // operands themselves stay: some elements are formed term by term).  With 4 x 4
+    // blocks L's wait for Z (slot 0) and S's for U (slot 1, the others' too).
+    int tags = 0, tag_of[2] = {0, 0};
+    auto digits = [&](const lnv_plan *pl, void *a, void *b, int slot = 1, bool again = false) {
         DigScratch d;
         if (plan_digits(pl, nsf, pr)) {
             d.a = nsf == 9 ? ws + wl.D : a;
             d.b = nsf == 9 ? ws + wl.E : b;
             d.head = (int *)(ws + wl.head);
+            d.slot = slot;
+            d.have_a = again && nsf == 4 && tag_of[slot];
+            d.tag_b = tags += 2;
+            if (!d.have_a) tag_of[slot] = d.tag_b;
+            d.tag_a = tag_of[slot];
         }
         return d;
     };
     auto product = [&](const lnv_plan *pl, const DigScratch &d, const void *A, const void *B1, const void *B2, void *C1,
-                       void *C2) { return multiply2(ctx, pl, nsf, pr, A, B1, B2, C1, C2, d.a ? &d : nullptr); };
-    void *D = ws + wl.D;
+                       void *C2, bool whole = false) {
+        return multiply2(ctx, pl, nsf, pr, A, B1, B2, C1, C2, d.a ? &d : nullptr, whole);
+    };
+    void *D = ws + wl.D, *DL = ws + wl.V;
+    // with 4 x 4 blocks T's digits take U's place for Z: U is formed after Z then
+    const bool late_u = grad && nsf == 4 && plan_digits(sys->pl_z, nsf, pr);
     if (plan_digits(sys->pl_xy, nsf, pr) || plan_digits(sys->pl_tu, nsf, pr) || plan_digits(sys->pl_z, nsf, pr) ||
         plan_digits(sys->pl_q, nsf, pr) || plan_digits(sys->pl_w, nsf, pr))
-        LNV_CUDA(cudaMemsetAsync(ws + wl.head, 0, dig_zero_bytes(), ctx->stream));
+        LNV_CUDA(cudaMemsetAsync(ws + wl.head, 0, dig_zero_bytes(sys->n, nsf), ctx->stream));
     LNV_TRY(mark(0));
     // a1: X = L S, Y = L H (S's, then H's digits where T comes later)
-    LNV_TRY(product(sys->pl_xy, digits(sys->pl_xy, D, sys->P_sh->nnzb <= sys->P_t->nnzb ? T : ws + wl.E), L_dev, S_dev, H_dev, X, Y));
+    LNV_TRY(product(sys->pl_xy, digits(sys->pl_xy, DL, T, 0), L_dev, S_dev, H_dev, X, Y));
     LNV_TRY(mark(1));
     // a2: T = S X (= SLS), U = S Y (= SLH) (X's, then Y's digits where Z comes later)
     const DigScratch d_tu = digits(sys->pl_tu, D, Z);
-    if (grad) LNV_TRY(product(sys->pl_tu, d_tu, S_dev, X, Y, T, U));
+    if (grad && !late_u) LNV_TRY(product(sys->pl_tu, d_tu, S_dev, X, Y, T, U));
     else LNV_TRY(product(sys->pl_tu, d_tu, S_dev, X, nullptr, T, nullptr));
-    // Z and W on digits overwrite T, which dN_e/dL reads on L's pattern: its
-    // blocks wait in the output
-    const bool t_early = GN_dev && (plan_digits(sys->pl_z, nsf, pr) || (grad && plan_digits(sys->pl_w, nsf, pr)));
+    // the digits of Y (for U after Z) and of U (for W) overwrite T, which dN_e/dL
+    // reads on L's pattern: its blocks wait in the output
+    const bool t_early = GN_dev && grad && (late_u || plan_digits(sys->pl_w, nsf, pr));
     if (t_early) LNV_TRY(sub_blocks(ctx, sys->P_l, sys->sub_lt, nsf, pr, T, GN_dev));
     LNV_TRY(mark(2));
-    // a3: Z = L T (= LSLS) on R_X (T's digits replace T)
-    DigScratch d_z = digits(sys->pl_z, D, T);
-    d_z.b_finite = plan_digits(sys->pl_tu, nsf, pr);
-    LNV_TRY(product(sys->pl_z, d_z, L_dev, T, nullptr, Z, nullptr));
+    // a3: Z = L T (= LSLS) on R_X (T's digits where U comes later)
+    LNV_TRY(product(sys->pl_z, digits(sys->pl_z, DL, ws + wl.U, 0, true), L_dev, T, nullptr, Z, nullptr));
     LNV_TRY(mark(3));
     // a4: Tr[XY], Tr[ZY], Tr[XX], Tr[ZX] -> E, N_e per system
     const void *ta[4] = {X, Z, X, Z}, *tb[4] = {Y, Y, X, X};
@@ -843,13 +867,17 @@ lnv_status lnv_energy_grad(lnv_ctx *ctx, lnv_system *sys, const void *S_dev, con
     LNV_TRY(reduce_rows(ctx, rows, sys->n, 4, sys->n_seg, sys->seg_off_dev, out_dev, 6, 2));
     LNV_TRY(lnv_combine(ctx, sys->n_seg, out_dev));
     LNV_TRY(mark(4));
+    sys->profiled_u = sys->profile && late_u;
+    if (late_u) {
+        LNV_TRY(product(sys->pl_tu, digits(sys->pl_tu, D, T, 1, true), S_dev, Y, nullptr, U, nullptr, true));
+        if (sys->profile) LNV_CUDA(cudaEventRecord(sys->ev_u, ctx->stream));
+    }
     if (grad) {
         // a6: Q = H Z (= HLSLS) on R_L;  a5: W = X^T U^T (= SLHLS) on R_L
         // (Z's and X's digits where Y was, U's where T was)
-        const DigScratch d_q = digits(sys->pl_q, D, Y);
-        LNV_TRY(product(sys->pl_q, d_q, H_dev, Z, nullptr, Q, nullptr));
+        LNV_TRY(product(sys->pl_q, digits(sys->pl_q, D, Y), H_dev, Z, nullptr, Q, nullptr));
         // V = S Z (= SLSLS) on R_L has the patterns of Q = H Z
-        if (GN_dev) LNV_TRY(product(sys->pl_q, d_q, S_dev, Z, nullptr, V, nullptr));
+        if (GN_dev) LNV_TRY(product(sys->pl_q, digits(sys->pl_q, D, Y), S_dev, Z, nullptr, V, nullptr));
         LNV_TRY(mark(5));
         LNV_TRY(product(sys->pl_w, digits(sys->pl_w, Y, T), X, U, nullptr, W, nullptr));
         LNV_TRY(mark(6));

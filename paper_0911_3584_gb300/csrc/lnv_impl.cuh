@@ -287,19 +287,21 @@ lnv_status tile_plan_build(lnv_ctx *ctx, lnv_plan *pl, size_t budget_bytes);
 // Kernel 11 on FP64 values with NSF = 4 and kernel 10 on FP64 values with NSF = 9
 // (umma64.cu; the latter in plans whose owner named the values).  Their operands
 // are split into digits in buffers of dig_bytes(A), dig_bytes(B) and
-// dig_head_bytes(n); with NSF = 4 b may be B itself with op(B) = B^T (B is then
-// overwritten).  The first dig_zero_bytes() of head are zero before the first product
-// of an evaluation; with b = B, b_finite says that B is a result of such a product (whose
-// infinities are known).
+// dig_head_bytes(n), which hold neither operand.  The first dig_zero_bytes(n) of head
+// are zero before the first product of an evaluation.  head holds what is known of the
+// rows of two operands op(A) (slot) and of one op(B), under a tag for each that is split:
+// tag_a, tag_b, and with two products tag_b + 1.  have_a: a and head hold op(A)'s digits
+// and rows, split in an earlier product under tag_a.
 constexpr int kDigRec = 12;  // ints of a CTA's schedule record
 struct DigScratch {
     void *a = nullptr, *b = nullptr;
     int *head = nullptr;
-    bool b_finite = false;
+    int slot = 0, tag_a = 1, tag_b = 1;
+    bool have_a = false;
 };
 size_t dig_bytes(const lnv_pattern *P, int nsf);
 size_t dig_head_bytes(int64_t n, int nsf);
-size_t dig_zero_bytes();
+size_t dig_zero_bytes(int64_t n, int nsf);
 // Schedule of its CTAs over the tiles of meta: whole waves, then one record per CTA.
 struct DigSchedule {
     int waves = 0;
@@ -313,9 +315,8 @@ inline bool plan_digits(const lnv_plan *pl, int nsf, lnv_prec prec)
     return prec == LNV_FP64 && pl->tt.meta && (pl->trans_b || pl->B->symmetric) &&
            ((pl->mode == 11 && nsf == 4) || (pl->mode == 10 && nsf == 9 && pl->tc.G == kTc9dG));
 }
-// reuse_a: a and head hold A's digits and magnitudes of the call before.
 lnv_status launch_umma64(lnv_ctx *ctx, const lnv_plan *pl, int nsf, bool upper, const void *A, const void *B, void *C,
-                         const DigScratch &s, bool reuse_a);
+                         const DigScratch &s);
 void tile_plan_free(TilePlan *tt);
 lnv_status scan_exclusive(cudaStream_t st, const int64_t *in, int64_t n, int64_t *out);
 void group_plan_free(GroupPlan *gp);
@@ -327,9 +328,10 @@ lnv_status multiply(lnv_ctx *ctx, const lnv_plan *plan, int nsf, lnv_prec prec, 
                     const void *B, void *C);
 // Two products sharing A and the patterns of B and C: C1 = A B1, C2 = A B2.
 // dig: the digit buffers of a plan with plan_digits (null: taken from the context's pool
-// for the call).
+// for the call).  whole: C1 is not symmetric, also where the plan's first output is.
 lnv_status multiply2(lnv_ctx *ctx, const lnv_plan *plan, int nsf, lnv_prec prec, const void *A,
-                     const void *B1, const void *B2, void *C1, void *C2, const DigScratch *dig = nullptr);
+                     const void *B1, const void *B2, void *C1, void *C2, const DigScratch *dig = nullptr,
+                     bool whole = false);
 
 // Vectors on value arrays (minimize.cu): out = a x + b y (x, y not read when
 // their factor is 0); *out_dev = x.y in FP64 (fixed-order reduction)

@@ -1,6 +1,6 @@
 """FP64 digit products (kernel 11 on FP64 values, kernel 10 on those of 9 x 9 systems) at the limits of their
 operands: NaN and infinities met while the operands are split, results at the ends of the exponent range, buffers of
-the digits that outlive a call."""
+the digits that outlive a call, operands whose elements differ by many powers of two."""
 from fractions import Fraction
 
 import numpy as np
@@ -173,4 +173,141 @@ def test_truncation_below_the_range_of_s(cuda_device, nsf):
         assert abs(out[0, 0].item() - ref["E"]) <= 1e-12 * abs(ref["E"])
         assert abs(out[0, 1].item() - ref["Ne"]) <= 1e-12 * abs(ref["Ne"])
         assert rel_fro(G.cpu().numpy(), ref["G"]) <= 1e-13
+    assert ctx.device_status() == 0
+
+
+def _elementwise(ctx, n_atoms, a, b, ta, tb):
+    """(|C - ref|, K |A||B|) of a product on the full pattern of n_atoms atoms, ref and |A||B| in long double."""
+    n = n_atoms
+    P = Pattern.build(ctx, np.random.default_rng(0).uniform(0, 5.0, size=(n, 3)), np.array([30.0, 30.0, 30.0]), 14.9)
+    assert P.nnzb == n * n
+    blocks = [np.ascontiguousarray(v.reshape(n, 4, n, 4).transpose(0, 2, 1, 3)).reshape(n * n, 4, 4) for v in
+              (a.T if ta else a, b.T if tb else b)]
+    plan = Plan(ctx, P, P, P, trans_a=ta, trans_b=tb)
+    plan.set_kernel("tensor-tile")
+    C = plan.multiply(*(to_dev(v, torch.float64, ctx.device) for v in blocks)).cpu().numpy()
+    C = C.reshape(n, n, 4, 4).transpose(0, 2, 1, 3).reshape(4 * n, 4 * n)
+    A, B = a.astype(np.longdouble), b.astype(np.longdouble)
+    return np.abs(C - A @ B), 4 * n * (np.abs(A) @ np.abs(B))
+
+
+@pytest.mark.parametrize("ta", [False, True])
+@pytest.mark.parametrize("tb", [False, True])
+@pytest.mark.parametrize("spread", [0, 5, 7, 20, 40, 60, 500])
+def test_inner_index_of_any_scale(ctx, spread, ta, tb):
+    """A D times D^-1 B with D of powers of two over a wide range: the bound K 2^-53 |A||B| of a plain FP64 sum, element
+    by element.  The digits' bound is K 2^-53 max|row of A| max|column of B|, with the largest elements at most 2^4
+    apart from those that they meet (the rest is formed term by term); 260 normal terms have |A||B| of about 166 and
+    max max of at most 16, so that bound is below 2^4 16 / 166 < 2 times the plain sum's: 4 is allowed."""
+    rng = np.random.default_rng(spread)
+    d = 2.0 ** np.round(spread * rng.uniform(-0.5, 0.5, size=260))
+    err, kab = _elementwise(ctx, 65, rng.standard_normal((260, 260)) * d, rng.standard_normal((260, 260)) / d[:, None],
+                            ta, tb)
+    assert np.all(err <= 4 * 2.0 ** -53 * kab), np.max(err / kab) / 2.0 ** -53
+
+
+@pytest.mark.parametrize("tb", [False, True])
+def test_large_element_that_meets_nothing(ctx, tb):
+    """Rows whose largest element, by 2^60, multiplies a row of zeros of B; columns likewise: the rest is exact."""
+    rng = np.random.default_rng(1)
+    a, b = rng.standard_normal((2, 36, 36))
+    a[:, 5] *= 2.0 ** 60
+    b[5] = 0.0
+    b[17] *= 2.0 ** 60
+    a[:, 17] = 0.0
+    err, kab = _elementwise(ctx, 9, a, b, False, tb)
+    assert np.all(err <= 2.0 ** -53 * kab), np.max(err / kab) / 2.0 ** -53
+
+
+def _rescaled(M, d, power):
+    """Blocks ij of M times d_i^power on their rows and d_j^power on their columns (d [n, nsf])."""
+    rows = np.repeat(np.arange(M["rp"].size - 1), np.diff(M["rp"]))
+    return M["val"] * (d[rows] ** power)[:, :, None] * (d[M["col"]] ** power)[:, None, :]
+
+
+@pytest.mark.parametrize("nsf", [4, 9])
+@pytest.mark.parametrize("spread", [0, 4, 10, 20, 40, 60])
+def test_evaluation_does_not_depend_on_the_scale_of_basis_functions(ctx, nsf, spread):
+    """S -> D S D, H -> D H D, L -> D^-1 L D^-1 with powers of two: E, N_e and the traces stay, dE/dL becomes D G D."""
+    rng = np.random.default_rng(spread)
+    if nsf == 4:
+        w, S, H, L = workload(2, 4, 6.6, 8.0, 5)
+        pos, cell, r = w["pos"], w["cell"], (6.6, 8.0)
+    else:
+        from synth import si_diamond_positions, sym_block_values
+        pos, cell = si_diamond_positions(2, rng)
+        pos, r = np.ascontiguousarray(pos[:43]), (4.0, 6.0)
+        pat = {k: oracle.pattern(pos, cell, c) for k, c in (("S", r[0]), ("H", r[0]), ("L", r[1]))}
+        S, H, L = (oracle.csr(*pat[k], sym_block_values(*pat[k], pos, cell, 9, k, rng)) for k in "SHL")
+    ref = oracle.lnv_energy_grad(pos, cell, *r, S, H, L, grad=True, grad_ne=True)
+    d = 2.0 ** np.round(spread * rng.uniform(-0.5, 0.5, size=(pos.shape[0], nsf)))
+    sysm = System(ctx, nsf, "fp64", pos, cell, *r)
+    out, G, GN = sysm.energy_grad(*(to_dev(_rescaled(M, d, p), torch.float64, ctx.device) for M, p in
+                                    ((S, 1.0), (H, 1.0), (L, -1.0))), grad_ne=True)
+    back = [_rescaled(dict(L, val=g.cpu().numpy()), d, -1.0) for g in (G, GN)]
+    assert abs(out[0, 0].item() - ref["E"]) <= 1e-12 * abs(ref["E"])
+    assert abs(out[0, 1].item() - ref["Ne"]) <= 1e-12 * abs(ref["Ne"])
+    assert rel_fro(back[0], ref["G"]) <= 1e-12
+    assert rel_fro(back[1], ref["GN"]) <= 1e-12
+    assert ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("bad", ["nan", "scale"])
+@pytest.mark.parametrize("nsf", [4, 9])
+def test_one_system_of_a_batch_does_not_touch_the_others(ctx, nsf, bad):
+    """A NaN in one system, or one of badly scaled basis functions: the bits of the others stay (groups of atoms
+    that the products take together span the systems)."""
+    rng = np.random.default_rng(4)
+    pos = [rng.uniform(0, 8.0, size=(n, 3)) for n in (21, 13, 18)]
+    cell, off = [40.0, 40.0, 40.0], [0, 21, 34, 52]
+    sysm = System(ctx, nsf, "fp64", np.concatenate(pos), [cell] * 3, 4.0, 5.0, seg_off=off)
+    dev = ctx.device
+
+    def vals(P, scale):
+        rp, col, tr = P.row_ptr.cpu(), P.col.cpu().long(), P.tr.cpu()
+        v = scale * torch.from_numpy(rng.standard_normal((P.nnzb, nsf, nsf)))
+        v = 0.5 * (v + v[tr].transpose(1, 2))
+        row = torch.repeat_interleave(torch.arange(P.n), rp[1:] - rp[:-1])
+        v[row == col] += torch.eye(nsf, dtype=torch.float64)
+        return v, row
+
+    S, row = vals(sysm.P_sh, 0.05)
+    H, _ = vals(sysm.P_sh, 0.3)
+    L, _ = vals(sysm.P_l, 0.02)
+    out0, G0 = sysm.energy_grad(S.to(dev), H.to(dev), L.to(dev))
+    mid = (row >= 21) & (row < 34)
+    if bad == "nan":
+        H[int(mid.nonzero()[3]), 1, 2] = float("nan")
+    else:
+        d = 2.0 ** torch.from_numpy(np.round(30 * rng.uniform(size=(52, nsf))))
+        S[mid] = (S * d[row][:, :, None] * d[sysm.P_sh.col.cpu().long()][:, None, :])[mid]
+    out, G = sysm.energy_grad(S.to(dev), H.to(dev), L.to(dev))
+    rp = sysm.P_l.row_ptr.cpu()
+    keep = torch.cat([torch.arange(int(rp[21])), torch.arange(int(rp[34]), sysm.P_l.nnzb)]).to(dev)
+    assert torch.equal(out[[0, 2]], out0[[0, 2]])
+    assert torch.equal(G[keep], G0[keep])
+    assert not torch.equal(out[1], out0[1])
+
+
+@pytest.mark.parametrize("digits", ["XY", "TU", "Z", "Q", "W"])
+@pytest.mark.parametrize("other", ["push", "pull", "group", "group-sparse", "triples"])
+@pytest.mark.parametrize("mirror", [True, False])
+def test_one_stage_on_digits_beside_plain_ones(ctx, digits, other, mirror):
+    """U is formed after Z when T's digits take its place, on the kernel of T and U, and is not symmetric as T is."""
+    w, S, H, L = workload(2, 4, 4.0, 5.0, 3)
+    ref = oracle.lnv_energy_grad(w["pos"], w["cell"], 4.0, 5.0, S, H, L, grad=True, grad_ne=True)
+    sysm = System(ctx, 4, "fp64", w["pos"], w["cell"], 4.0, 5.0)
+    for st in ("XY", "TU", "Z", "Q", "W"):
+        sysm.set_stage_kernel(st, "tensor-tile" if st == digits else other)
+    sysm.set_mirror(mirror)
+    sysm.profile(True)
+    vals = [to_dev(M["val"], torch.float64, ctx.device) for M in (S, H, L)]
+    for grad in (True, False):
+        out, G, GN = sysm.energy_grad(*vals, grad=grad, grad_ne=True)
+        assert abs(out[0, 0].item() - ref["E"]) <= 1e-12 * abs(ref["E"])
+        assert abs(out[0, 1].item() - ref["Ne"]) <= 1e-12 * abs(ref["Ne"])
+        assert rel_fro(GN.cpu().numpy(), ref["GN"]) <= 1e-13
+        if grad:
+            assert rel_fro(G.cpu().numpy(), ref["G"]) <= 1e-13
+            assert all(v > 0 for v in sysm.stage_ms().values())
     assert ctx.device_status() == 0
