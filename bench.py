@@ -894,8 +894,8 @@ def main():
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
         "data": "synthetic",
         "config": {"workload": WORKLOAD, "atoms": w_atoms(), "nsf": NSF, "r_sh": R_SH, "r_l": R_L,
-                   "precision": "FP32 block products and accumulation; FP64 traces, E, N_e and "
-                                "gradient combination",
+                   "precision": "FP32 block products and accumulation; FP64 sums of traces, E and N_e; "
+                                "gradient combined at FP64 accuracy",
                    "l2": "flushed between timed steps (256 MB write, outside the timed events)",
                    "parallelism": f"replicas x{world} (independent systems)"},
         "gflops": round(r32["flops"] / (r32["ms_per_step"] * 1e-3) / 1e9, 1),

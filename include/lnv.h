@@ -67,8 +67,9 @@ typedef int lnv_status;
  * depend on the scale of the basis functions.  Single elements far below those of their
  * row and column hold fewer bits; lnv_system_set_stage_kernel selects plain products.
  * LNV_FP32: values stored and multiplied in FP32 with FP32 accumulation of
- * the block products; traces, energies and the gradient combination are
- * accumulated in FP64 from the FP32 operands. */
+ * the block products; energies and the sums of the traces are accumulated in
+ * FP64 (the products of a block pair in FP32), and the gradient is combined from
+ * the FP32 operands with no less than FP64's accuracy and range. */
 typedef enum { LNV_FP64 = 0, LNV_FP32 = 1 } lnv_prec;
 
 /* Operand flags of lnv_plan_product: use the block transpose of A or B,
