@@ -203,7 +203,7 @@ lnv_status lnv_ctx_create(int device, void *cuda_stream, lnv_ctx **out)
     c->sm_count = v;
     cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
     c->smem_optin = (size_t)v;
-    cudaError_t e = cudaMalloc(&c->dev_status, sizeof(int));
+    cudaError_t e = dev_alloc(&c->dev_status, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->dev_status, 0, sizeof(int));
     if (e != cudaSuccess) {
         cudaFree(c->dev_status);
@@ -300,8 +300,8 @@ lnv_status lnv_pattern_from_csr(lnv_ctx *ctx, int64_t n, const int64_t *row_ptr_
         set_error("pattern block count %lld out of range", (long long)nnzb);
         return LNV_ERR_PATTERN;
     }
-    if (e == cudaSuccess) e = cudaMalloc(&p->row_ptr, sizeof(int64_t) * (n + 1));
-    if (e == cudaSuccess) e = cudaMalloc(&p->col, sizeof(int32_t) * std::max<int64_t>(nnzb, 1));
+    if (e == cudaSuccess) e = dev_alloc(&p->row_ptr, sizeof(int64_t) * (n + 1));
+    if (e == cudaSuccess) e = dev_alloc(&p->col, sizeof(int32_t) * std::max<int64_t>(nnzb, 1));
     if (e == cudaSuccess) e = cudaMemcpyAsync(p->row_ptr, row_ptr_dev, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToDevice, ctx->stream);
     if (e == cudaSuccess && nnzb > 0) {
         LNV_ARG(col_dev, "null columns");
@@ -388,7 +388,7 @@ lnv_status lnv_bsr_multiply(lnv_ctx *ctx, const lnv_plan *plan, int nsf, lnv_pre
         cudaFree(ctx->prod_scratch);
         ctx->prod_scratch = nullptr;
         ctx->prod_scratch_bytes = 0;
-        LNV_CUDA(cudaMalloc(&ctx->prod_scratch, bytes));
+        LNV_CUDA(dev_alloc(&ctx->prod_scratch, bytes));
         ctx->prod_scratch_bytes = bytes;
     }
     LNV_TRY(multiply(ctx, plan, nsf, prec, A_dev, B_dev, ctx->prod_scratch));
@@ -471,9 +471,9 @@ lnv_status lnv_system_create_truncated(lnv_ctx *ctx, int nsf, lnv_prec prec, con
     // W = X^T U^T = SLHLS is symmetric: only its upper triangle is formed
     SYS_TRY(pattern_upper(ctx, s->P_l, &s->P_lu));
     SYS_TRY(plan_create(ctx, s->P_x, s->P_t, s->P_lu, LNV_TRANS_A | LNV_TRANS_B, &s->pl_w, nsf, prec));
-    cudaError_t e = cudaMalloc(&s->sub_lt, sizeof(int64_t) * std::max<int64_t>(s->P_l->nnzb, 1));
-    if (e == cudaSuccess) e = cudaMalloc(&s->w_map, sizeof(int64_t) * std::max<int64_t>(s->P_l->nnzb, 1));
-    if (e == cudaSuccess) e = cudaMalloc(&s->seg_off_dev, sizeof(int64_t) * (n_seg + 1));
+    cudaError_t e = dev_alloc(&s->sub_lt, sizeof(int64_t) * std::max<int64_t>(s->P_l->nnzb, 1));
+    if (e == cudaSuccess) e = dev_alloc(&s->w_map, sizeof(int64_t) * std::max<int64_t>(s->P_l->nnzb, 1));
+    if (e == cudaSuccess) e = dev_alloc(&s->seg_off_dev, sizeof(int64_t) * (n_seg + 1));
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(s->seg_off_dev, off.data(), sizeof(int64_t) * (n_seg + 1), cudaMemcpyHostToDevice, ctx->stream);
     if (e != cudaSuccess) {
@@ -597,8 +597,8 @@ lnv_status lnv_system_autotune(lnv_ctx *ctx, lnv_system *sys, const void *S_dev,
     const WsLayout wl = ws_layout(sys, 1);
     void *G = nullptr;
     double *out = nullptr;
-    LNV_CUDA(cudaMalloc(&G, (size_t)sys->P_l->nnzb * sys->nsf * sys->nsf * elem_size(sys->prec) + 16));
-    cudaError_t e = cudaMalloc(&out, sizeof(double) * 6 * (size_t)sys->n_seg);
+    LNV_CUDA(dev_alloc(&G, (size_t)sys->P_l->nnzb * sys->nsf * sys->nsf * elem_size(sys->prec) + 16));
+    cudaError_t e = dev_alloc(&out, sizeof(double) * 6 * (size_t)sys->n_seg);
     if (e != cudaSuccess) {
         cudaFree(G);
         set_error("autotune allocation: %s", cudaGetErrorString(e));
@@ -757,7 +757,7 @@ lnv_status lnv_energy_grad_host(lnv_ctx *ctx, lnv_system *sys, const void *S_hos
     const size_t n_out = align256(sizeof(double) * 6 * (size_t)sys->n_seg);
     if (!sys->io_dev) {
         // S, H, L, G, out, each on a 256-byte boundary
-        cudaError_t e = cudaMalloc(&sys->io_dev, 2 * n_sh + 2 * n_l + n_out);
+        cudaError_t e = dev_alloc(&sys->io_dev, 2 * n_sh + 2 * n_l + n_out);
         if (e != cudaSuccess) {
             sys->io_dev = nullptr;
             set_error("host-evaluation buffers: %s", cudaGetErrorString(e));
@@ -798,7 +798,7 @@ lnv_status lnv_energy_grad(lnv_ctx *ctx, lnv_system *sys, const void *S_dev, con
             sys->own_ws_bytes = 0;
             // the largest layout (with gradient) so later calls never reallocate
             size_t need = ws_layout(sys, 1).total;
-            LNV_CUDA(cudaMalloc(&sys->own_ws, need));
+            LNV_CUDA(dev_alloc(&sys->own_ws, need));
             sys->own_ws_bytes = need;
         }
         ws = (unsigned char *)sys->own_ws;

@@ -115,7 +115,7 @@ lnv_status upload(const std::vector<X> &h, X **d, size_t *bytes)
 {
     *d = nullptr;
     if (h.empty()) return LNV_OK;
-    LNV_CUDA(cudaMalloc(d, sizeof(X) * h.size()));
+    LNV_CUDA(dev_alloc(d, sizeof(X) * h.size()));
     LNV_CUDA(cudaMemcpy(*d, h.data(), sizeof(X) * h.size(), cudaMemcpyHostToDevice));
     *bytes += sizeof(X) * h.size();
     return LNV_OK;
@@ -301,8 +301,8 @@ static lnv_status group_plan_lists(lnv_ctx *ctx, lnv_plan *pl, int G, size_t bud
     // hit counts per (group, j) -> offsets of the hit lists (the tensor-core kernels read neither)
     if (s == LNV_OK && j_off[ng] > 0 && !jmajor) {
         int64_t *cnt = nullptr;
-        cudaError_t e = cudaMalloc(&cnt, sizeof(int64_t) * (size_t)j_off[ng]);
-        if (e == cudaSuccess) e = cudaMalloc(&gp.hoff, sizeof(int64_t) * (size_t)(j_off[ng] + 1));
+        cudaError_t e = dev_alloc(&cnt, sizeof(int64_t) * (size_t)j_off[ng]);
+        if (e == cudaSuccess) e = dev_alloc(&gp.hoff, sizeof(int64_t) * (size_t)(j_off[ng] + 1));
         if (e == cudaSuccess) {
             k_hits<<<(unsigned)ng, 128, 0, ctx->stream>>>(gp.k_off, gp.k_list, gp.j_off, gp.j_list, B->row_ptr,
                                                          B->col, pl->trans_b, cnt, nullptr, nullptr, nullptr);
@@ -347,7 +347,7 @@ lnv_status group_plan_build_into(lnv_ctx *ctx, lnv_plan *pl, int G, size_t budge
             set_error("row-group position table needs %zu bytes, over the %zu budget", need, budget_bytes);
             return LNV_ERR_UNSUPPORTED;
         }
-        LNV_CUDA(cudaMalloc(&gp.bidx, need));
+        LNV_CUDA(dev_alloc(&gp.bidx, need));
         LNV_CUDA(cudaMemsetAsync(gp.bidx, 0xFF, need, ctx->stream));
         if (gp.jmajor)
             k_bidx_t<<<(unsigned)ng, 256, 0, ctx->stream>>>(gp.k_off, gp.k_list, gp.j_off, gp.j_list, gp.bidx_off,
@@ -365,8 +365,13 @@ lnv_status group_plan_build_into(lnv_ctx *ctx, lnv_plan *pl, int G, size_t budge
             set_error("row-group hit lists need %zu bytes, over the %zu budget", need, budget_bytes);
             return LNV_ERR_UNSUPPORTED;
         }
-        LNV_CUDA(cudaMalloc(&gp.hk, sizeof(uint16_t) * (size_t)gp.hits));
-        LNV_CUDA(cudaMalloc(&gp.hp, sizeof(int32_t) * (size_t)gp.hits));
+        // both or neither: lists that are there are not built again
+        LNV_CUDA(dev_alloc(&gp.hp, sizeof(int32_t) * (size_t)gp.hits));
+        if (const cudaError_t e = dev_alloc(&gp.hk, sizeof(uint16_t) * (size_t)gp.hits)) {
+            cudaFree(gp.hp);
+            gp.hp = nullptr;
+            LNV_CUDA(e);
+        }
         k_hits<<<(unsigned)ng, 128, 0, ctx->stream>>>(gp.k_off, gp.k_list, gp.j_off, gp.j_list, B->row_ptr, B->col,
                                                      pl->trans_b, nullptr, gp.hoff, gp.hk, gp.hp);
         LNV_LAUNCHED();

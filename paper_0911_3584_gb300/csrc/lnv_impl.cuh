@@ -38,6 +38,19 @@ void set_error(const char *fmt, ...);
         }                                                    \
     } while (0)
 
+// cudaMalloc whose failure is in its result alone: a refused allocation that is reported or
+// survived (by smaller tables, another kernel) is not found again by a later launch check.
+template <class T>
+inline cudaError_t dev_alloc(T **p, size_t bytes)
+{
+    const cudaError_t e = cudaMalloc((void **)p, bytes);
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        cudaGetLastError();
+    }
+    return e;
+}
+
 // Launch check after a kernel<<<>>>; also counts the library's kernel launches.
 void count_launch();
 #define LNV_LAUNCHED()                   \

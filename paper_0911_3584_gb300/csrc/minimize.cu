@@ -95,7 +95,7 @@ lnv_status ctx_scratch(lnv_ctx *ctx, size_t n_doubles, double **out)
         cudaFree(ctx->scratch);
         ctx->scratch = nullptr;
         ctx->scratch_n = 0;
-        LNV_CUDA(cudaMalloc(&ctx->scratch, sizeof(double) * n_doubles));
+        LNV_CUDA(dev_alloc(&ctx->scratch, sizeof(double) * n_doubles));
         ctx->scratch_n = n_doubles;
     }
     *out = ctx->scratch;
@@ -189,9 +189,9 @@ struct Minimiser {
 
     lnv_status alloc(size_t h_bytes)
     {
-        LNV_CUDA(cudaMalloc(&Hp, std::max<size_t>(h_bytes, 16)));
-        for (void **p : {&G, &D, &g_old, &Lt}) LNV_CUDA(cudaMalloc(p, std::max<size_t>(bytes, 16)));
-        LNV_CUDA(cudaMalloc(&dev, sizeof(double) * 8));
+        LNV_CUDA(dev_alloc(&Hp, std::max<size_t>(h_bytes, 16)));
+        for (void **p : {&G, &D, &g_old, &Lt}) LNV_CUDA(dev_alloc(p, std::max<size_t>(bytes, 16)));
+        LNV_CUDA(dev_alloc(&dev, sizeof(double) * 8));
         return LNV_OK;
     }
 

@@ -298,8 +298,8 @@ lnv_status scan_exclusive(cudaStream_t st, const int64_t *in, int64_t n, int64_t
         return LNV_OK;
     }
     int64_t *sums = nullptr, *offs = nullptr;
-    LNV_CUDA(cudaMalloc(&sums, sizeof(int64_t) * nb));
-    LNV_CUDA(cudaMalloc(&offs, sizeof(int64_t) * (nb + 1)));
+    LNV_CUDA(dev_alloc(&sums, sizeof(int64_t) * nb));
+    LNV_CUDA(dev_alloc(&offs, sizeof(int64_t) * (nb + 1)));
     k_scan_block<<<(unsigned)nb, T, 0, st>>>(in, n, out, sums);
     LNV_LAUNCHED();
     lnv_status s = LNV_OK;
@@ -358,14 +358,14 @@ lnv_status pattern_finish(lnv_ctx *ctx, lnv_pattern *p, bool sort_rows)
         LNV_LAUNCHED();
     }
     int64_t nn = std::max<int64_t>(p->nnzb, 1);
-    LNV_CUDA(cudaMalloc(&p->row, sizeof(int32_t) * nn));
-    LNV_CUDA(cudaMalloc(&p->tr, sizeof(int64_t) * nn));
+    LNV_CUDA(dev_alloc(&p->row, sizeof(int32_t) * nn));
+    LNV_CUDA(dev_alloc(&p->tr, sizeof(int64_t) * nn));
     if (p->n > 0) {
         k_row_of<<<(unsigned)((p->n + 255) / 256), 256, 0, st>>>(p->row_ptr, p->n, p->row);
         LNV_LAUNCHED();
     }
     int *d_asym = nullptr;
-    LNV_CUDA(cudaMalloc(&d_asym, sizeof(int)));
+    LNV_CUDA(dev_alloc(&d_asym, sizeof(int)));
     LNV_CUDA(cudaMemsetAsync(d_asym, 0, sizeof(int), st));
     if (p->nnzb > 0) {
         k_transpose_map<<<(unsigned)((p->nnzb + 255) / 256), 256, 0, st>>>(
@@ -434,16 +434,16 @@ lnv_status pattern_build_impl(lnv_ctx *ctx, const double *pos, int n_seg, const 
         }                                         \
     } while (0)
     int64_t nn = std::max<int64_t>(n, 1);
-    STEP(cudaMalloc(&d_segs, sizeof(SegGrid) * n_seg));
+    STEP(dev_alloc(&d_segs, sizeof(SegGrid) * n_seg));
     STEP(cudaMemcpyAsync(d_segs, segs.data(), sizeof(SegGrid) * n_seg, cudaMemcpyHostToDevice, st));
-    STEP(cudaMalloc(&atom_seg, sizeof(int32_t) * nn));
-    STEP(cudaMalloc(&atom_bin, sizeof(int64_t) * nn));
-    STEP(cudaMalloc(&bin_atoms, sizeof(int32_t) * nn));
-    STEP(cudaMalloc(&bin_count, sizeof(unsigned long long) * nbins));
-    STEP(cudaMalloc(&bin_count64, sizeof(int64_t) * nbins));
-    STEP(cudaMalloc(&bin_start, sizeof(int64_t) * (nbins + 1)));
-    STEP(cudaMalloc(&row_cnt, sizeof(int64_t) * nn));
-    STEP(cudaMalloc(&p->row_ptr, sizeof(int64_t) * (n + 1)));
+    STEP(dev_alloc(&atom_seg, sizeof(int32_t) * nn));
+    STEP(dev_alloc(&atom_bin, sizeof(int64_t) * nn));
+    STEP(dev_alloc(&bin_atoms, sizeof(int32_t) * nn));
+    STEP(dev_alloc(&bin_count, sizeof(unsigned long long) * nbins));
+    STEP(dev_alloc(&bin_count64, sizeof(int64_t) * nbins));
+    STEP(dev_alloc(&bin_start, sizeof(int64_t) * (nbins + 1)));
+    STEP(dev_alloc(&row_cnt, sizeof(int64_t) * nn));
+    STEP(dev_alloc(&p->row_ptr, sizeof(int64_t) * (n + 1)));
     STEP(cudaMemsetAsync(bin_count, 0, sizeof(unsigned long long) * nbins, st));
     unsigned g = (unsigned)((n + 255) / 256);
     if (n > 0) {
@@ -473,7 +473,7 @@ lnv_status pattern_build_impl(lnv_ctx *ctx, const double *pos, int n_seg, const 
         set_error("pattern has %lld blocks; at most 2^31-1 are supported", (long long)nnzb);
         return fail(LNV_ERR_UNSUPPORTED);
     }
-    STEP(cudaMalloc(&p->col, sizeof(int32_t) * std::max<int64_t>(nnzb, 1)));
+    STEP(dev_alloc(&p->col, sizeof(int32_t) * std::max<int64_t>(nnzb, 1)));
     if (n > 0) {
         k_neighbours<<<g, 256, 0, st>>>(pos, n, d_segs, atom_seg, atom_bin, bin_start, bin_atoms,
                                          cutoff * cutoff, nullptr, p->row_ptr, p->col);
@@ -502,8 +502,8 @@ lnv_status pattern_upper(lnv_ctx *ctx, const lnv_pattern *P, lnv_pattern **out)
             if (P->h_col[q] >= i) col.push_back(P->h_col[q]);
         rp[i + 1] = (int64_t)col.size();
     }
-    cudaError_t e = cudaMalloc(&u->row_ptr, sizeof(int64_t) * (P->n + 1));
-    if (e == cudaSuccess) e = cudaMalloc(&u->col, sizeof(int32_t) * std::max<size_t>(col.size(), 1));
+    cudaError_t e = dev_alloc(&u->row_ptr, sizeof(int64_t) * (P->n + 1));
+    if (e == cudaSuccess) e = dev_alloc(&u->col, sizeof(int32_t) * std::max<size_t>(col.size(), 1));
     if (e == cudaSuccess) e = cudaMemcpy(u->row_ptr, rp.data(), sizeof(int64_t) * (P->n + 1), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !col.empty())
         e = cudaMemcpy(u->col, col.data(), sizeof(int32_t) * col.size(), cudaMemcpyHostToDevice);
@@ -575,7 +575,7 @@ lnv_status pattern_remap(lnv_ctx *ctx, const lnv_pattern *from, const lnv_patter
 lnv_status pattern_validate(lnv_ctx *ctx, const lnv_pattern *p)
 {
     int *bad = nullptr;
-    LNV_CUDA(cudaMalloc(&bad, sizeof(int)));
+    LNV_CUDA(dev_alloc(&bad, sizeof(int)));
     LNV_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), ctx->stream));
     if (p->n > 0) {
         k_validate<<<(unsigned)((p->n + 255) / 256), 256, 0, ctx->stream>>>(p->row_ptr, p->col, p->n, bad);

@@ -36,7 +36,7 @@ lnv_status fma_rate(lnv_ctx *ctx, int iters, double *tflops)
 {
     const int blocks = ctx->sm_count * 8, threads = 256;
     T *out = nullptr;
-    LNV_CUDA(cudaMalloc(&out, sizeof(T) * (size_t)blocks * threads));
+    LNV_CUDA(dev_alloc(&out, sizeof(T) * (size_t)blocks * threads));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);

@@ -120,12 +120,12 @@ lnv_status triple_plan_build(lnv_ctx *ctx, lnv_plan *pl, size_t budget_bytes)
         for (auto &x : th) x.join();
     }
     size_t bytes = 0;
-    cudaError_t e = cudaMalloc(&tp.item_cb, sizeof(int32_t) * std::max<size_t>(1, items.size()));
-    if (e == cudaSuccess) e = cudaMalloc(&tp.t_off, sizeof(int64_t) * (size_t)(C->nnzb + 1));
+    cudaError_t e = dev_alloc(&tp.item_cb, sizeof(int32_t) * std::max<size_t>(1, items.size()));
+    if (e == cudaSuccess) e = dev_alloc(&tp.t_off, sizeof(int64_t) * (size_t)(C->nnzb + 1));
     if (e == cudaSuccess && !items.empty())
         e = cudaMemcpy(tp.item_cb, items.data(), sizeof(int32_t) * items.size(), cudaMemcpyHostToDevice);
     int64_t *cnt = nullptr;
-    if (e == cudaSuccess) e = cudaMalloc(&cnt, sizeof(int64_t) * std::max<int64_t>(1, C->nnzb));
+    if (e == cudaSuccess) e = dev_alloc(&cnt, sizeof(int64_t) * std::max<int64_t>(1, C->nnzb));
     if (e != cudaSuccess) {
         cudaFree(cnt);
         triple_plan_free(&tp);
@@ -191,7 +191,7 @@ lnv_status triple_plan_build(lnv_ctx *ctx, lnv_plan *pl, size_t budget_bytes)
         s = LNV_ERR_PATTERN;
     }
     if (s == LNV_OK && total > 0) {
-        if (cudaMalloc(&tp.tri, sizeof(int2) * (size_t)total) != cudaSuccess) {
+        if (dev_alloc(&tp.tri, sizeof(int2) * (size_t)total) != cudaSuccess) {
             set_error("triple-list plan: allocation of %lld triples failed", (long long)total);
             s = LNV_ERR_OOM;
         } else {
@@ -216,7 +216,7 @@ lnv_status triple_plan_build(lnv_ctx *ctx, lnv_plan *pl, size_t budget_bytes)
             if (C->h_col[(size_t)items[t]] >= row_of[(size_t)items[t]]) up.push_back((int32_t)t);
         tp.n_up = (int64_t)up.size();
         if (!up.empty()) {
-            if (cudaMalloc(&tp.up, sizeof(int32_t) * up.size()) != cudaSuccess ||
+            if (dev_alloc(&tp.up, sizeof(int32_t) * up.size()) != cudaSuccess ||
                 cudaMemcpy(tp.up, up.data(), sizeof(int32_t) * up.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
                 set_error("triple-list plan: allocation of the upper-triangle items failed");
                 s = LNV_ERR_OOM;

@@ -407,7 +407,7 @@ __global__ void k_tile_lists(int64_t n_items, const int2 *__restrict__ items, co
 template <typename X>
 cudaError_t upload_vec(const std::vector<X> &h, X **d)
 {
-    cudaError_t e = cudaMalloc(d, sizeof(X) * std::max<size_t>(1, h.size()));
+    cudaError_t e = dev_alloc(d, sizeof(X) * std::max<size_t>(1, h.size()));
     if (e == cudaSuccess && !h.empty()) e = cudaMemcpy(*d, h.data(), sizeof(X) * h.size(), cudaMemcpyHostToDevice);
     return e;
 }
@@ -474,8 +474,8 @@ lnv_status tile_plan_build(lnv_ctx *ctx, lnv_plan *pl, size_t budget_bytes)
     cudaError_t e = upload_vec(items, &tt.items);
     if (e == cudaSuccess) e = upload_vec(up, &tt.up);
     int64_t *cnt = nullptr;
-    if (e == cudaSuccess) e = cudaMalloc(&cnt, sizeof(int64_t) * std::max<int64_t>(1, tt.n_items));
-    if (e == cudaSuccess) e = cudaMalloc(&tt.ck_off, sizeof(int64_t) * (size_t)(tt.n_items + 1));
+    if (e == cudaSuccess) e = dev_alloc(&cnt, sizeof(int64_t) * std::max<int64_t>(1, tt.n_items));
+    if (e == cudaSuccess) e = dev_alloc(&tt.ck_off, sizeof(int64_t) * (size_t)(tt.n_items + 1));
     if (e != cudaSuccess) {
         cudaFree(cnt);
         tile_plan_free(&tt);
@@ -504,8 +504,8 @@ lnv_status tile_plan_build(lnv_ctx *ctx, lnv_plan *pl, size_t budget_bytes)
         s = LNV_ERR_UNSUPPORTED;
     }
     if (s == LNV_OK && listed > 0) {
-        if (cudaMalloc(&tt.ck_apos, sizeof(int32_t) * tab_g * (size_t)listed) != cudaSuccess ||
-            cudaMalloc(&tt.ck_blk, sizeof(int32_t) * tab_cols * (size_t)listed) != cudaSuccess) {
+        if (dev_alloc(&tt.ck_apos, sizeof(int32_t) * tab_g * (size_t)listed) != cudaSuccess ||
+            dev_alloc(&tt.ck_blk, sizeof(int32_t) * tab_cols * (size_t)listed) != cudaSuccess) {
             set_error("kernel 11 tile plan: allocation of %lld listed k's failed", (long long)listed);
             s = LNV_ERR_OOM;
         } else {
