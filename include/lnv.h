@@ -221,10 +221,12 @@ lnv_status lnv_plan_product(lnv_ctx *ctx, const lnv_pattern *A, const lnv_patter
  * Kernels 9-13 need value arrays 16-byte aligned (else LNV_ERR_UNSUPPORTED
  * from the multiply).
  * The default is 3 when at least half of the table's candidates hit, else 4,
- * when the tables fit a third of the free device memory; 4 x 4 blocks are then
- * multiplied on the listed triples (7) where fewer than an eighth of the (k, j)
- * candidates hit, until a kernel is selected by hand.  The products of a system
- * with 4 x 4 blocks begin with 11 (FP64), 7 or 8 (FP32). */
+ * when the tables fit a third of the free device memory.  Where fewer than an
+ * eighth of the (k, j) candidates hit, a plan of lnv_plan_product lists its triples
+ * too (8 bytes each, while they fit) and multiplies 4 x 4 blocks of either type on
+ * kernel 7 until a kernel is selected by hand; *mode is then the kernel of the
+ * other block sizes.  The products of a system know their values: with 4 x 4
+ * blocks they begin with 11 (FP64), 7 or 8 (FP32), with 9 x 9 blocks in FP64 with 10. */
 lnv_status lnv_plan_info(const lnv_plan *plan, int64_t *triples, int *mode);
 /* Number of product kernels (0 .. LNV_NUM_KERNELS - 1). */
 #define LNV_NUM_KERNELS 14
