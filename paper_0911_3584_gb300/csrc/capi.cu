@@ -96,6 +96,8 @@ struct lnv_system {
     int profile = 0;
     int profiled_grad = 0;
     cudaEvent_t ev[kStages + 1] = {};
+    // FP64 products of 4 x 4 or 9 x 9 blocks may run on digits (the workspace has room for them)
+    bool digits = false;
     cudaEvent_t ev_u = nullptr;  // after U, where it is formed after Z (profiled_u)
     bool profiled_u = false;
 };
@@ -133,7 +135,7 @@ WsLayout ws_layout(const lnv_system *s, int with_grad)
     // (see lnv_energy_grad): those of S, H, Y and U to T, which they may not fit if T is
     // truncated, those of T to U, which is needed for this without the gradient too, and
     // those of L to V, which comes last.
-    const bool dig = (s->nsf == 4 || s->nsf == 9) && s->prec == LNV_FP64, dig9 = dig && s->nsf == 9, dig4 = dig && !dig9;
+    const bool dig = s->digits, dig9 = dig && s->nsf == 9, dig4 = dig && !dig9;
     const int64_t n_t = dig4 ? std::max({s->P_t->nnzb, s->P_x->nnzb, s->P_sh->nnzb}) : s->P_t->nnzb;
     L.T = take(n_t * bs);
     L.U = with_grad || dig4 ? take(s->P_t->nnzb * bs) : 0;
@@ -150,10 +152,41 @@ WsLayout ws_layout(const lnv_system *s, int with_grad)
     return L;
 }
 
+void free_plans(lnv_system *s)
+{
+    for (lnv_plan **p : {&s->pl_xy, &s->pl_tu, &s->pl_z, &s->pl_q, &s->pl_w}) {
+        plan_free(*p);
+        *p = nullptr;
+    }
+}
+
+// The five products' plans; nsf: the values' block size, or -1 for row groups whatever it is.
+lnv_status make_plans(lnv_ctx *ctx, lnv_system *s, int nsf, lnv_prec prec, bool exact_x)
+{
+    LNV_TRY(plan_create(ctx, s->P_l, s->P_sh, s->P_x, 0, &s->pl_xy, nsf, prec));
+    // T = SLS is symmetric when X = LS is exact (L symmetric): only its upper
+    // triangle is formed, the lower one mirrored.  With X truncated it is not.
+    LNV_TRY(plan_create(ctx, s->P_sh, s->P_x, s->P_t, exact_x ? LNV_SYM_C : 0, &s->pl_tu, nsf, prec));
+    // Z = L T: T = SLS is symmetric, so L T = L T^T; the transposed form lets
+    // the merge-join pull read T's row j in order instead of through tr.
+    LNV_TRY(plan_create(ctx, s->P_l, s->P_t, s->P_x, LNV_TRANS_B, &s->pl_z, nsf, prec));
+    LNV_TRY(plan_create(ctx, s->P_sh, s->P_x, s->P_l, 0, &s->pl_q, nsf, prec));
+    return plan_create(ctx, s->P_x, s->P_t, s->P_lu, LNV_TRANS_A | LNV_TRANS_B, &s->pl_w, nsf, prec);
+}
+
+// Do an evaluation's workspace and its S, H, L and G fit the free device memory?
+bool workspace_fits(const lnv_system *s)
+{
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return true;
+    const size_t bs = (size_t)s->nsf * s->nsf * elem_size(s->prec);
+    return ws_layout(s, 1).total + 2 * bs * (size_t)(s->P_sh->nnzb + s->P_l->nnzb) <= free_b;
+}
+
 void system_free(lnv_system *s)
 {
     if (!s) return;
-    plan_free(s->pl_xy); plan_free(s->pl_tu); plan_free(s->pl_z); plan_free(s->pl_q); plan_free(s->pl_w);
+    free_plans(s);
     pattern_free(s->P_sh); pattern_free(s->P_l); pattern_free(s->P_x); pattern_free(s->P_t);
     pattern_free(s->P_lu);
     cudaFree(s->w_map);
@@ -460,17 +493,17 @@ lnv_status lnv_system_create_truncated(lnv_ctx *ctx, int nsf, lnv_prec prec, con
     SYS_TRY(pattern_build_impl(ctx, pos_dev, n_seg, off.data(), cells_host, r_l, &s->P_l));
     SYS_TRY(pattern_build_impl(ctx, pos_dev, n_seg, off.data(), cells_host, r_x, &s->P_x));
     SYS_TRY(pattern_build_impl(ctx, pos_dev, n_seg, off.data(), cells_host, r_t, &s->P_t));
-    SYS_TRY(plan_create(ctx, s->P_l, s->P_sh, s->P_x, 0, &s->pl_xy, nsf, prec));
-    // T = SLS is symmetric when X = LS is exact (L symmetric): only its upper
-    // triangle is formed, the lower one mirrored.  With X truncated it is not.
-    SYS_TRY(plan_create(ctx, s->P_sh, s->P_x, s->P_t, r_x >= r_l + r_sh ? LNV_SYM_C : 0, &s->pl_tu, nsf, prec));
-    // Z = L T: T = SLS is symmetric, so L T = L T^T; the transposed form lets
-    // the merge-join pull read T's row j in order instead of through tr.
-    SYS_TRY(plan_create(ctx, s->P_l, s->P_t, s->P_x, LNV_TRANS_B, &s->pl_z, nsf, prec));
-    SYS_TRY(plan_create(ctx, s->P_sh, s->P_x, s->P_l, 0, &s->pl_q, nsf, prec));
     // W = X^T U^T = SLHLS is symmetric: only its upper triangle is formed
     SYS_TRY(pattern_upper(ctx, s->P_l, &s->P_lu));
-    SYS_TRY(plan_create(ctx, s->P_x, s->P_t, s->P_lu, LNV_TRANS_A | LNV_TRANS_B, &s->pl_w, nsf, prec));
+    s->digits = (nsf == 4 || nsf == 9) && prec == LNV_FP64;
+    SYS_TRY(make_plans(ctx, s, nsf, prec, r_x >= r_l + r_sh));
+    if (s->digits && !workspace_fits(s)) {
+        // no room for digits beside the intermediates: the kernels and the workspace of a
+        // system without them
+        s->digits = false;
+        free_plans(s);
+        SYS_TRY(make_plans(ctx, s, -1, prec, r_x >= r_l + r_sh));
+    }
     cudaError_t e = dev_alloc(&s->sub_lt, sizeof(int64_t) * std::max<int64_t>(s->P_l->nnzb, 1));
     if (e == cudaSuccess) e = dev_alloc(&s->w_map, sizeof(int64_t) * std::max<int64_t>(s->P_l->nnzb, 1));
     if (e == cudaSuccess) e = dev_alloc(&s->seg_off_dev, sizeof(int64_t) * (n_seg + 1));
@@ -821,9 +854,10 @@ lnv_status lnv_energy_grad(lnv_ctx *ctx, lnv_system *sys, const void *S_dev, con
     // operands themselves stay: some elements are formed term by term).  With 4 x 4
     // blocks L's wait for Z (slot 0) and S's for U (slot 1, the others' too).
     int tags = 0, tag_of[2] = {0, 0};
+    auto has_digits = [&](const lnv_plan *pl) { return sys->digits && plan_digits(pl, nsf, pr); };
     auto digits = [&](const lnv_plan *pl, void *a, void *b, int slot = 1, bool again = false) {
         DigScratch d;
-        if (plan_digits(pl, nsf, pr)) {
+        if (has_digits(pl)) {
             d.a = nsf == 9 ? ws + wl.D : a;
             d.b = nsf == 9 ? ws + wl.E : b;
             d.head = (int *)(ws + wl.head);
@@ -841,9 +875,9 @@ lnv_status lnv_energy_grad(lnv_ctx *ctx, lnv_system *sys, const void *S_dev, con
     };
     void *D = ws + wl.D, *DL = ws + wl.V;
     // with 4 x 4 blocks T's digits take U's place for Z: U is formed after Z then
-    const bool late_u = grad && nsf == 4 && plan_digits(sys->pl_z, nsf, pr);
-    if (plan_digits(sys->pl_xy, nsf, pr) || plan_digits(sys->pl_tu, nsf, pr) || plan_digits(sys->pl_z, nsf, pr) ||
-        plan_digits(sys->pl_q, nsf, pr) || plan_digits(sys->pl_w, nsf, pr))
+    const bool late_u = grad && nsf == 4 && has_digits(sys->pl_z);
+    if (has_digits(sys->pl_xy) || has_digits(sys->pl_tu) || has_digits(sys->pl_z) || has_digits(sys->pl_q) ||
+        has_digits(sys->pl_w))
         LNV_CUDA(cudaMemsetAsync(ws + wl.head, 0, dig_zero_bytes(sys->n, nsf), ctx->stream));
     LNV_TRY(mark(0));
     // a1: X = L S, Y = L H (S's, then H's digits where T comes later)
@@ -855,7 +889,7 @@ lnv_status lnv_energy_grad(lnv_ctx *ctx, lnv_system *sys, const void *S_dev, con
     else LNV_TRY(product(sys->pl_tu, d_tu, S_dev, X, nullptr, T, nullptr));
     // the digits of Y (for U after Z) and of U (for W) overwrite T, which dN_e/dL
     // reads on L's pattern: its blocks wait in the output
-    const bool t_early = GN_dev && grad && (late_u || plan_digits(sys->pl_w, nsf, pr));
+    const bool t_early = GN_dev && grad && (late_u || has_digits(sys->pl_w));
     if (t_early) LNV_TRY(sub_blocks(ctx, sys->P_l, sys->sub_lt, nsf, pr, T, GN_dev));
     LNV_TRY(mark(2));
     // a3: Z = L T (= LSLS) on R_X (T's digits where U comes later)

@@ -257,7 +257,8 @@ lnv_status pattern_submap(lnv_ctx *ctx, const lnv_pattern *sub, const lnv_patter
 // Product internals (mult.cu)
 // flags: LNV_TRANS_A, LNV_TRANS_B, LNV_SYM_C (the first output of the plan's
 // products is symmetric; C's pattern must be symmetric)
-// nsf, prec: those of the values, where the caller knows them (nsf = 0: unknown).
+// nsf, prec: those of the values, where the caller knows them (nsf = 0: unknown; -1: the
+// row groups, and no triple lists beside them).
 lnv_status plan_create(lnv_ctx *ctx, const lnv_pattern *A, const lnv_pattern *B,
                        const lnv_pattern *C, int flags, lnv_plan **out, int nsf = 0, lnv_prec prec = LNV_FP64);
 // The strict lower triangle of a matrix on the symmetric pattern P set from its
