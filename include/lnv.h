@@ -63,8 +63,9 @@ typedef int lnv_status;
  * or a column that is not finite, or whose largest element meets no element of the
  * other operand within 2^-4 of the largest of its own column or row (as when the
  * inner index is badly scaled), is formed term by term in FP64 all the same: so in the
- * largest element of every row and column both bounds are of one size, and E, N_e and G do not
- * depend on the scale of the basis functions.  Single elements far below those of their
+ * largest element of every row and column both bounds are of one size.  A system's
+ * products take the norms of the basis functions (from S's diagonal) out of the inner
+ * index first: E, N_e and G do not depend on them.  Single elements far below those of their
  * row and column hold fewer bits; lnv_system_set_stage_kernel selects plain products.
  * LNV_FP32: values stored and multiplied in FP32 with FP32 accumulation of
  * the block products; energies and the sums of the traces are accumulated in

@@ -251,6 +251,8 @@ void pattern_free(lnv_pattern *p);
 lnv_status pattern_upper(lnv_ctx *ctx, const lnv_pattern *P, lnv_pattern **out);
 lnv_status pattern_upper_map(lnv_ctx *ctx, const lnv_pattern *P, const lnv_pattern *U, int64_t *map_dev);
 // position map of every block of `sub` inside `super` (both sorted), -1 if absent
+// Positions of a range pattern's diagonal blocks.
+lnv_status pattern_diagonal(lnv_ctx *ctx, const lnv_pattern *p, int64_t *out_dev);
 lnv_status pattern_submap(lnv_ctx *ctx, const lnv_pattern *sub, const lnv_pattern *super,
                           int64_t *map_dev);
 
@@ -312,10 +314,15 @@ struct DigScratch {
     int *head = nullptr;
     int slot = 0, tag_a = 1, tag_b = 1;
     bool have_a = false;
+    // inner index of op(A) times 2^d and that of op(B) times 2^-d (1), the other way
+    // round (-1), d from dig_begin; or neither (0)
+    int balance = 0;
 };
 size_t dig_bytes(const lnv_pattern *P, int nsf);
 size_t dig_head_bytes(int64_t n, int nsf);
 size_t dig_zero_bytes(int64_t n, int nsf);
+// Begin of an evaluation: head's zeros, and the basis functions' norms from S's diagonal blocks.
+lnv_status dig_begin(lnv_ctx *ctx, int *head, int64_t n, int nsf, const int64_t *diag, const void *S);
 // Schedule of its CTAs over the tiles of meta: whole waves, then one record per CTA.
 struct DigSchedule {
     int waves = 0;

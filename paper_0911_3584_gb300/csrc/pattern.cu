@@ -225,6 +225,20 @@ __global__ void k_transpose_map(const int64_t *__restrict__ row_ptr, const int32
     if (q < 0) atomicOr(asym, 1);
 }
 
+// Position of each row's diagonal block (range patterns hold every one).
+__global__ void k_diagonal(const int64_t *__restrict__ rp, const int32_t *__restrict__ col, int64_t n, int64_t *out)
+{
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    int64_t lo = rp[i], hi = rp[i + 1] - 1;
+    while (lo < hi) {
+        const int64_t mid = lo + ((hi - lo) >> 1);
+        if (col[mid] < i) lo = mid + 1;
+        else hi = mid;
+    }
+    out[i] = lo;
+}
+
 __global__ void k_submap(const int64_t *__restrict__ s_rp, const int32_t *__restrict__ s_col,
                          const int32_t *__restrict__ s_row, int64_t nnzb,
                          const int64_t *__restrict__ p_rp, const int32_t *__restrict__ p_col,
@@ -549,6 +563,14 @@ lnv_status pattern_submap(lnv_ctx *ctx, const lnv_pattern *sub, const lnv_patter
     if (sub->nnzb == 0) return LNV_OK;
     k_submap<<<(unsigned)((sub->nnzb + 255) / 256), 256, 0, ctx->stream>>>(
         sub->row_ptr, sub->col, sub->row, sub->nnzb, super->row_ptr, super->col, map_dev);
+    LNV_LAUNCHED();
+    return LNV_OK;
+}
+
+lnv_status pattern_diagonal(lnv_ctx *ctx, const lnv_pattern *p, int64_t *out_dev)
+{
+    if (p->n == 0) return LNV_OK;
+    k_diagonal<<<(unsigned)((p->n + 255) / 256), 256, 0, ctx->stream>>>(p->row_ptr, p->col, p->n, out_dev);
     LNV_LAUNCHED();
     return LNV_OK;
 }

@@ -311,3 +311,54 @@ def test_one_stage_on_digits_beside_plain_ones(ctx, digits, other, mirror):
             assert rel_fro(G.cpu().numpy(), ref["G"]) <= 1e-13
             assert all(v > 0 for v in sysm.stage_ms().values())
     assert ctx.device_status() == 0
+
+
+def test_each_order_of_digits(ctx):
+    """Rows of A with one digit per element, of order s, and columns of B with one of order t: products with s + t <= 5
+    are exact, those of 6 and 7 are added in units of 2^-6 of order 5 (2^-58 here), so no order is missing or at a
+    wrong place.  The largest elements, of the scales, meet zeros in these rows and columns, and are met in others (A's
+    at inner index 0, B's at 1), so that the digits are kept."""
+    rng = np.random.default_rng(2)
+    n = 6
+    a, b = np.zeros((4 * n, 4 * n)), np.zeros((4 * n, 4 * n))
+    da, db = (rng.integers(-60, 61, size=(7, 4 * n - 2)) for _ in "ab")
+    for s in range(7):  # the largest is 1: digit s has the weight 2^(-6 - 8 s)
+        a[s, 0], a[s, 2:] = 1.0, da[s] * 2.0 ** (-6 - 8 * s)
+        b[1, s], b[2:, s] = 1.0, db[s] * 2.0 ** (-6 - 8 * s)
+    b[0, 10] = a[10, 1] = 1.0
+    P = Pattern.build(ctx, np.random.default_rng(0).uniform(0, 5.0, size=(n, 3)), np.array([30.0, 30.0, 30.0]), 14.9)
+    blocks = [np.ascontiguousarray(v.reshape(n, 4, n, 4).transpose(0, 2, 1, 3)).reshape(n * n, 4, 4) for v in (a, b)]
+    plan = Plan(ctx, P, P, P)
+    plan.set_kernel("tensor-tile")
+    C = plan.multiply(*(to_dev(v, torch.float64, ctx.device) for v in blocks)).cpu().numpy()
+    C = C.reshape(n, n, 4, 4).transpose(0, 2, 1, 3).reshape(4 * n, 4 * n)
+    want = (da @ db.T) * 2.0 ** (-12.0 - 8.0 * np.add.outer(np.arange(7), np.arange(7)))
+    order = np.add.outer(np.arange(7), np.arange(7))
+    C = C[:7, :7]
+    assert np.array_equal(C[order <= 5], want[order <= 5])
+    low = (order == 6) | (order == 7)
+    assert np.all(np.abs(C[low] - want[low]) <= 2.0 ** -59) and np.abs(want[order == 7]).min() > 2.0 ** -58
+    assert np.all(C[order > 7] == 0.0)  # not formed
+
+
+@pytest.mark.parametrize("nsf", [4, 9])
+@pytest.mark.parametrize("spread", [10, 60, 300])
+def test_norms_of_basis_functions_change_no_bit(ctx, nsf, spread):
+    """S -> D S D, H -> D H D, L -> D^-1 L D^-1 with powers of two and S_kk = 1 before: the digits are those of the
+    normalised functions, so E, N_e and the traces have the same bits, and dE/dL and dN_e/dL with D taken out."""
+    rng = np.random.default_rng(nsf)
+    from synth import si_diamond_positions, sym_block_values
+    pos, cell = si_diamond_positions(2, rng)
+    pos, r = np.ascontiguousarray(pos[:43]), (4.0, 6.0)
+    pat = {k: oracle.pattern(pos, cell, c) for k, c in (("S", r[0]), ("H", r[0]), ("L", r[1]))}
+    M = {k: oracle.csr(*pat[k], sym_block_values(*pat[k], pos, cell, nsf, k, rng)) for k in "SHL"}
+    d = 2.0 ** np.round(spread * rng.uniform(-0.5, 0.5, size=(pos.shape[0], nsf)))
+    got = []
+    for dd in (np.ones_like(d), d):
+        sysm = System(ctx, nsf, "fp64", pos, cell, *r)
+        out, G, GN = sysm.energy_grad(*(to_dev(_rescaled(M[k], dd, p), torch.float64, ctx.device) for k, p in
+                                        (("S", 1.0), ("H", 1.0), ("L", -1.0))), grad_ne=True)
+        got.append([out.cpu().numpy()] + [_rescaled(dict(M["L"], val=g.cpu().numpy()), dd, -1.0) for g in (G, GN)])
+    for x, y in zip(*got):
+        assert np.array_equal(x, y)
+    assert ctx.device_status() == 0
