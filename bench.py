@@ -37,9 +37,12 @@ KERNEL_NAME = {"push": "k_push2", "pull": "k_pull", "pull-merge": "k_pull2", "gr
                "group-sparse": "k_grp (hit lists)", "group-pipe": "k_gw", "group-mma": "k_gmma",
                "triples": "k_tri", "group-pipe-half": "k_gw (half-width slices)",
                "tensor": "k_umma (tcgen05, 3xTF32)", "tensor9": "k_umma9 (tcgen05, 3xTF32, NSF = 9)",
-               "tensor-tile": "k_umma_tile (tcgen05, per-tile k lists; 3xTF32, FP64: k_umma64, FP16 digits)",
+               "tensor-tile": "k_umma_tile (tcgen05, 3xTF32, per-tile k lists)",
                "tensor-1pass": "k_umma (tcgen05, single-pass TF32)",
                "tensor-tile-1pass": "k_umma_tile (tcgen05, single-pass TF32)"}
+# the same kernel numbers on FP64 values
+KERNEL_NAME_FP64 = {"tensor9": "k_umma64 (tcgen05, FP16 digits of FP64 values, NSF = 9)",
+                    "tensor-tile": "k_umma64 (tcgen05, FP16 digits of FP64 values)"}
 TENSOR_KERNELS = ("tensor", "tensor9", "tensor-tile", "tensor-1pass", "tensor-tile-1pass")
 # the single-pass TF32 measurement: tcgen05 kernels 12 and 13 where 9 and 11 run
 SINGLE_PASS_KERNELS = {"XY": "triples", "TU": "tensor-tile-1pass", "Z": "tensor-1pass",
@@ -259,6 +262,10 @@ def time_path(ctx, w, prec, steps, warmup, dist, kernels=None):
     return res
 
 
+def kernel_name(k, prec):
+    return KERNEL_NAME_FP64.get(k, KERNEL_NAME[k]) if prec == "fp64" else KERNEL_NAME[k]
+
+
 def measured_peaks():
     """The GPU's measured copy bandwidth and BF16 GEMM rate (MEASURED_PEAKS.json
     at the repository root), else fallback figures of 6.8 TB/s and 1.9
@@ -298,7 +305,7 @@ def roofline_tensor(res):
             continue
         ms = res["stage_ms"][st]
         achieved = res["flops_stage"][st] / (ms * 1e-3) / 1e12
-        out.append({"stage": st, "kernel": f"{KERNEL_NAME[k]} ({STAGE_KERNEL[st]})", "bound": "tensor",
+        out.append({"stage": st, "kernel": f"{kernel_name(k, res['prec'])} ({STAGE_KERNEL[st]})", "bound": "tensor",
                     "achieved": round(achieved, 3), "peak": round(tf32, 1), "unit": "TFLOP/s",
                     "frac": round(achieved / tf32, 4), "traffic": ncu_traffic(st, res["prec"]),
                     "kernel_ms": round(ms, 4),
@@ -321,7 +328,7 @@ def roofline(res, fma_tflops=None):
     kern = res["kernels"][stage]
     out = {"bound": "alu", "achieved": round(achieved, 4), "unit": "TFLOP/s",
            "traffic": ncu_traffic(stage, prec),
-           "kernel": f"{KERNEL_NAME[kern]} ({STAGE_KERNEL[stage]})"
+           "kernel": f"{kernel_name(kern, prec)} ({STAGE_KERNEL[stage]})"
                      + (" on T's upper triangle, then k_mirror_lower" if stage == "TU" and res["t_mirrored"]
                         else ""),
            "stage": stage, "kernel_ms": round(ms, 4),
