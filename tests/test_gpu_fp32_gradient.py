@@ -32,3 +32,15 @@ def test_fp32_gradient_is_combined_in_more_than_fp32(ctx, nsf, h, l):
     _, G = sysm.energy_grad(m["S"], m["H"], m["L"])
     assert np.isfinite(want)
     assert G[0, 0, 0].item() == want, (G[0, 0, 0].item(), want, u, q, w)
+
+
+@pytest.mark.parametrize("nsf", [1, 4])
+@pytest.mark.parametrize("h", [1.9 * 2.0 ** 127, -1.9 * 2.0 ** 127, float("inf"), float("nan")])
+def test_fp32_gradient_that_leaves_the_range(ctx, nsf, h):
+    """G = 12 h (l - l^2) beyond the range of FP32 is infinite, of its sign; NaN and infinite terms give NaN."""
+    sysm = System(ctx, nsf, "fp32", np.zeros((1, 3)) + 1.0, [40.0, 40.0, 40.0], 4.0, 5.0)
+    m = {k: torch.zeros((1, nsf, nsf), dtype=torch.float32, device=ctx.device) for k in "SHL"}
+    m["S"][0, 0, 0], m["H"][0, 0, 0], m["L"][0, 0, 0] = 1.0, h, 0.5
+    _, G = sysm.energy_grad(m["S"], m["H"], m["L"])
+    want = np.copysign(np.inf, h) if np.isfinite(h) else np.nan
+    assert np.array_equal(G[0, 0, 0].item(), want, equal_nan=True)
