@@ -362,3 +362,34 @@ def test_norms_of_basis_functions_change_no_bit(ctx, nsf, spread):
     for x, y in zip(*got):
         assert np.array_equal(x, y)
     assert ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("bad", [0.0, np.nan, np.inf])
+@pytest.mark.parametrize("zero", ["a", "b", "both", "some"])
+def test_zero_rows_and_columns(ctx, zero, bad):
+    """Operands of zeros, whole or in part: zeros against finite elements, NaN against others, as term by term."""
+    rng = np.random.default_rng(3)
+    P = Pattern.build(ctx, rng.uniform(0, 9.0, size=(42, 3)), np.array([20.0, 20.0, 20.0]), 6.0)
+    v = {k: rng.standard_normal((P.nnzb, 4, 4)) for k in "ab"}
+    rows = np.repeat(np.arange(42), np.diff(P.row_ptr.cpu().numpy()))
+    for k in "ab":
+        if zero in (k, "both"):
+            v[k][:] = 0.0
+        elif zero == "some":
+            v[k][rows % 3 == 1] = 0.0
+            v[k][P.col.cpu().numpy() % 5 == 2] = 0.0
+            v[k][:, 2] = 0.0
+    if bad != 0.0:
+        v["a"][7, 1, 2] = bad
+        v["b"][100, 0, 3] = bad
+    out = {}
+    for kernel in ("triples", "tensor-tile"):
+        plan = Plan(ctx, P, P, P, trans_b=True)
+        plan.set_kernel(kernel)
+        out[kernel] = plan.multiply(*(to_dev(v[k], torch.float64, ctx.device) for k in "ab")).cpu().numpy()
+    ref, C = out["triples"], out["tensor-tile"]
+    assert np.array_equal(np.isnan(ref), np.isnan(C)) and np.array_equal(ref == 0.0, C == 0.0)
+    fine = np.isfinite(ref)
+    assert np.array_equal(ref[~fine & ~np.isnan(ref)], C[~fine & ~np.isnan(ref)])
+    assert np.linalg.norm(C[fine] - ref[fine]) <= 1e-14 * np.linalg.norm(ref[fine])
+    assert ctx.device_status() == 0
