@@ -96,7 +96,7 @@ struct lnv_system {
     int profile = 0;
     int profiled_grad = 0;
     cudaEvent_t ev[kStages + 1] = {};
-    int64_t *diag_sh = nullptr;  // positions of P_sh's diagonal blocks (systems with digits)
+    int64_t *diag_sh = nullptr, *diag_l = nullptr;  // positions of the diagonal blocks (systems with digits)
     // FP64 products of 4 x 4 or 9 x 9 blocks may run on digits (the workspace has room for them)
     bool digits = false;
     cudaEvent_t ev_u = nullptr;  // after U, where it is formed after Z (profiled_u)
@@ -193,6 +193,7 @@ void system_free(lnv_system *s)
     cudaFree(s->w_map);
     cudaFree(s->sub_lt);
     cudaFree(s->diag_sh);
+    cudaFree(s->diag_l);
     cudaFree(s->seg_off_dev);
     cudaFree(s->own_ws);
     cudaFree(s->io_dev);
@@ -509,6 +510,7 @@ lnv_status lnv_system_create_truncated(lnv_ctx *ctx, int nsf, lnv_prec prec, con
     cudaError_t e = dev_alloc(&s->sub_lt, sizeof(int64_t) * std::max<int64_t>(s->P_l->nnzb, 1));
     if (e == cudaSuccess) e = dev_alloc(&s->w_map, sizeof(int64_t) * std::max<int64_t>(s->P_l->nnzb, 1));
     if (e == cudaSuccess && s->digits) e = dev_alloc(&s->diag_sh, sizeof(int64_t) * std::max<int64_t>(s->n, 1));
+    if (e == cudaSuccess && s->digits) e = dev_alloc(&s->diag_l, sizeof(int64_t) * std::max<int64_t>(s->n, 1));
     if (e == cudaSuccess) e = dev_alloc(&s->seg_off_dev, sizeof(int64_t) * (n_seg + 1));
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(s->seg_off_dev, off.data(), sizeof(int64_t) * (n_seg + 1), cudaMemcpyHostToDevice, ctx->stream);
@@ -519,6 +521,7 @@ lnv_status lnv_system_create_truncated(lnv_ctx *ctx, int nsf, lnv_prec prec, con
     }
     SYS_TRY(pattern_submap(ctx, s->P_l, s->P_t, s->sub_lt));
     if (s->digits) SYS_TRY(pattern_diagonal(ctx, s->P_sh, s->diag_sh));
+    if (s->digits) SYS_TRY(pattern_diagonal(ctx, s->P_l, s->diag_l));
     SYS_TRY(pattern_upper_map(ctx, s->P_l, s->P_lu, s->w_map));
 #undef SYS_TRY
     e = cudaStreamSynchronize(ctx->stream);
@@ -886,7 +889,7 @@ lnv_status lnv_energy_grad(lnv_ctx *ctx, lnv_system *sys, const void *S_dev, con
     const bool late_u = grad && nsf == 4 && has_digits(sys->pl_z);
     if (has_digits(sys->pl_xy) || has_digits(sys->pl_tu) || has_digits(sys->pl_z) || has_digits(sys->pl_q) ||
         has_digits(sys->pl_w))
-        LNV_TRY(dig_begin(ctx, (int *)(ws + wl.head), sys->n, nsf, sys->diag_sh, S_dev));
+        LNV_TRY(dig_begin(ctx, (int *)(ws + wl.head), sys->n, nsf, sys->diag_sh, S_dev, sys->P_l, sys->diag_l, L_dev));
     LNV_TRY(mark(0));
     // a1: X = L S, Y = L H (S's, then H's digits where T comes later)
     LNV_TRY(product(sys->pl_xy, digits(sys->pl_xy, DL, T, 0), L_dev, S_dev, H_dev, X, Y));

@@ -321,8 +321,10 @@ struct DigScratch {
 size_t dig_bytes(const lnv_pattern *P, int nsf);
 size_t dig_head_bytes(int64_t n, int nsf);
 size_t dig_zero_bytes(int64_t n, int nsf);
-// Begin of an evaluation: head's zeros, and the basis functions' norms from S's diagonal blocks.
-lnv_status dig_begin(lnv_ctx *ctx, int *head, int64_t n, int nsf, const int64_t *diag, const void *S);
+// Begin of an evaluation: head's zeros, the basis functions' norms from S's diagonal blocks,
+// and the functions that L does not use.
+lnv_status dig_begin(lnv_ctx *ctx, int *head, int64_t n, int nsf, const int64_t *diag_s, const void *S,
+                     const lnv_pattern *PL, const int64_t *diag_l, const void *L);
 // Schedule of its CTAs over the tiles of meta: whole waves, then one record per CTA.
 struct DigSchedule {
     int waves = 0;

@@ -393,3 +393,35 @@ def test_zero_rows_and_columns(ctx, zero, bad):
     assert np.array_equal(ref[~fine & ~np.isnan(ref)], C[~fine & ~np.isnan(ref)])
     assert np.linalg.norm(C[fine] - ref[fine]) <= 1e-14 * np.linalg.norm(ref[fine])
     assert ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("nsf", [4, 9])
+@pytest.mark.parametrize("unused", ["one", "all but one", "all", "diagonal only"])
+def test_functions_that_l_does_not_use(ctx, nsf, unused):
+    """Rows and columns of L that are zero (or only its diagonal element is): E, N_e, G and dN_e/dL of the oracle; a NaN of
+    H at such a function still reaches E and G."""
+    rng = np.random.default_rng(nsf)
+    from synth import si_diamond_positions, sym_block_values
+    pos, cell = si_diamond_positions(2, rng)
+    pos, r = np.ascontiguousarray(pos[:43]), (4.0, 6.0)
+    pat = {k: oracle.pattern(pos, cell, c) for k, c in (("S", r[0]), ("H", r[0]), ("L", r[1]))}
+    M = {k: oracle.csr(*pat[k], sym_block_values(*pat[k], pos, cell, nsf, k, rng)) for k in "SHL"}
+    rows = np.repeat(np.arange(43), np.diff(M["L"]["rp"]))
+    L = M["L"]["val"]
+    dead = {"one": [2], "all but one": list(range(1, nsf)), "all": list(range(nsf)), "diagonal only": []}[unused]
+    L[:, dead, :] = 0.0
+    L[:, :, dead] = 0.0
+    if unused == "diagonal only":
+        L[np.ix_(rows == M["L"]["col"], [1], [1])] = 0.0
+    ref = oracle.lnv_energy_grad(pos, cell, *r, M["S"], M["H"], M["L"], grad=True, grad_ne=True)
+    sysm = System(ctx, nsf, "fp64", pos, cell, *r)
+    vals = [to_dev(M[k]["val"], torch.float64, ctx.device) for k in "SHL"]
+    out, G, GN = sysm.energy_grad(*vals, grad_ne=True)
+    assert abs(out[0, 0].item() - ref["E"]) <= 1e-12 * abs(ref["E"])
+    assert abs(out[0, 1].item() - ref["Ne"]) <= 1e-12 * abs(ref["Ne"])
+    assert rel_fro(G.cpu().numpy(), ref["G"]) <= 1e-13
+    assert rel_fro(GN.cpu().numpy(), ref["GN"]) <= 1e-13
+    vals[1][0, 2, 2] = float("nan")
+    out, G = sysm.energy_grad(*vals)
+    assert torch.isnan(out[0, 0]) and torch.isnan(G).any() and not torch.isnan(out[0, 1])
+    assert ctx.device_status() == 0
